@@ -51,11 +51,10 @@ FP64_PEAK_TFLOPS = 1.25
 
 
 def legendre_fp64_work(triples: int) -> float:
-    """FP64 work of one Legendre pass: 3 flops (one multiply, one FMA: the
-    rescaled three-term recurrence) per (ring pair, l, m) triple the kernel
-    runs.  The multiply occupies a full FMA slot, so the attainable peak for
-    this 1:1 mix is 3/4 of the FMA peak."""
-    return 3.0 * triples
+    """FP64 work of one Legendre pass: one FMA (2 flops) per (ring pair, l, m)
+    triple the kernel runs (the two-degree recurrence: two FMAs per two
+    degrees)."""
+    return 2.0 * triples
 
 
 class Clocks:
@@ -426,7 +425,7 @@ def main():
     fp = results["fp64"]
     M = fp["info"]["M"]
     flops = legendre_fp64_work(fp["info"]["leg_triples"])
-    peak = FP64_PEAK_TFLOPS * 0.75
+    peak = FP64_PEAK_TFLOPS
     traffic = {}
     prof = os.path.join(ROOT, "profiles", "legendre_traffic.json")
     if os.path.exists(prof):
@@ -442,15 +441,15 @@ def main():
     # launching stream (the adjoint stage includes the 0.3 ms partial-sum
     # reduction kernel).
     leg = {}
-    for kname, direction in (("legendre_synth_df_k", "synth"), ("legendre_adj_df_k", "adjoint")):
+    for kname, direction in (("leg2_synth_k", "synth"), ("leg2_adj_k", "adjoint")):
         t_leg = fp["stages"][direction]["legendre"] * 1e-3
         ach = flops / t_leg / 1e12
         leg[kname] = {"ms": t_leg * 1e3, "achieved": ach, "frac": ach / peak, "traffic": traffic.get(kname)}
     dom = max(leg, key=lambda k: leg[k]["ms"])
     roofline = {"bound": "alu", "achieved": leg[dom]["achieved"], "peak": peak, "unit": "TFLOP/s",
                 "frac": leg[dom]["frac"], "traffic": leg[dom]["traffic"],
-                "kernel": dom + ": FP64 recurrence (1 DMUL + 1 DFMA = 3 flops per triple) on the FP64 pipe; "
-                                "peak = 152 SMs x 2 FP64 FMA lanes/clk x 2.07 GHz x 3 flops / 2 slots (nominal; "
+                "kernel": dom + ": FP64 recurrence (2 DFMA = 4 flops per two triples) on the FP64 pipe; "
+                                "peak = 152 SMs x 2 FP64 FMA lanes/clk x 2.07 GHz x 2 flops (nominal; "
                                 "no FP64 figure in the measured peaks)",
                 "flops_per_launch": flops, "triples_per_launch": fp["info"]["leg_triples"],
                 "per_kernel": leg}
@@ -462,9 +461,9 @@ def main():
                "extrapolated": True,
                "sample": "%d seeded points (synthesis + adjoint over all orders), scaled by N/%d; "
                          "the direct sum is exactly linear in N" % (nsample, nsample)}
-    # synthesis: scale_alm_df, legendre_synth_df, poles_synth, theta DFT, column pass, row pass, interp_df;
-    # adjoint: spread_df, row pass, column pass, theta DFT, legendre_adj_df, adj_reduce_df
-    launches_per_step = 13
+    # synthesis: leg2_coef, leg2_synth, theta DFT, column pass, row pass, interp_df;
+    # adjoint: spread_df, row pass, column pass, theta DFT, leg2_adj, leg2_reduce
+    launches_per_step = 12
     line = {
         "metric": METRIC, "value": fp["ms"] / world, "unit": "ms", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": fp["ms"], "higher_is_better": False, "scaling": "weak",
@@ -790,7 +789,7 @@ def _kernel_hash() -> str:
     import hashlib
 
     h = hashlib.sha1()
-    for f in ("legendre.cu", "recurrence.cuh", "dfloat.cuh"):
+    for f in ("legendre.cu", "legendre2.cu", "recurrence.cuh", "dfloat.cuh"):
         with open(os.path.join(ROOT, "paper_2406_14542_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:12]

@@ -35,6 +35,25 @@ __device__ __forceinline__ void split_q(double q, float& qh, float& ql) {
   ql = __uint_as_float(__float_as_uint(__fmul_rn(r, sc)) | sign);
 }
 
+// The same with h rounded to nearest: |l| is at most half an ulp of h, so the
+// dropped product of two low words is a quarter as large as under split_q's
+// truncation and has either sign.  |q| < 2^-74 gives zero; |q| < 2^127.
+__device__ __forceinline__ void split_qr(double q, float& qh, float& ql) {
+  const int hi = __double2hiint(q);
+  const unsigned lo = (unsigned)__double2loint(q);
+  const unsigned sign = (unsigned)hi & 0x80000000u;
+  // add half of the 24th significant bit, keep the leading 24
+  const unsigned lr = lo + 0x10000000u;
+  const unsigned hr = (unsigned)hi + (lr < lo ? 1u : 0u);
+  const unsigned h = __funnelshift_l(lr, hr, 3) - ((unsigned)(1023 - 127) << 23);
+  // the remaining 29 bits as a signed integer, times 2^(e - 52)
+  const float r = __int2float_rn((int)(lo << 3) >> 3);
+  const unsigned sc = ((unsigned)hi << 3 & 0x7f800000u) - ((unsigned)((1023 - 127 + 52) & 0xff) << 23);
+  const bool in = ((unsigned)hi & 0x7ff00000u) >= ((unsigned)(1023 - 74) << 20);
+  qh = in ? __uint_as_float((h & 0x7fffffffu) | sign) : 0.0f;
+  ql = in ? __fmul_rn(r, __uint_as_float((sc & 0x7f800000u) | sign)) : 0.0f;
+}
+
 // (sh + sl) += (ah + al) * (qh + ql)
 __device__ __forceinline__ void df_mac(float& sh, float& sl, float ah, float al, float qh, float ql) {
   const float p = __fmul_rn(ah, qh);

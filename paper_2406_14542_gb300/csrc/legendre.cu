@@ -396,23 +396,11 @@ __global__ void scale_alm_df_k(const double* __restrict__ alm, const double* __r
   at[i] = r;
 }
 
-// q as a float pair: split off the FP64 chain's double, or the double-float
-// chain's own pair
-__device__ __forceinline__ void qsplit(const Chain& ch, float& qh, float& ql) { split_q(ch.q1, qh, ql); }
-__device__ __forceinline__ void qsplit(const DfChain& ch, float& qh, float& ql) {
-  qh = ch.q1.x;
-  ql = ch.q1.y;
+__device__ __forceinline__ void df_acc_step(float4& acc, const float4 av, const DfChain& ch) {
+  df_mac(acc.x, acc.y, av.x, av.y, ch.q1.x, ch.q1.y);
+  df_mac(acc.z, acc.w, av.z, av.w, ch.q1.x, ch.q1.y);
 }
 
-template <class CH>
-__device__ __forceinline__ void df_acc_step(float4& acc, const float4 av, const CH& ch) {
-  float qh, ql;
-  qsplit(ch, qh, ql);
-  df_mac(acc.x, acc.y, av.x, av.y, qh, ql);
-  df_mac(acc.z, acc.w, av.z, av.w, qh, ql);
-}
-
-template <class CH>
 __global__ void __launch_bounds__(128) legendre_synth_df_k(LegArgs a, const float4* __restrict__ at,
                                                            double2* __restrict__ G, int nitems) {
   const int lane = threadIdx.x & 31;
@@ -422,7 +410,7 @@ __global__ void __launch_bounds__(128) legendre_synth_df_k(LegArgs a, const floa
   item_of(a, it, m, blk);
   const int L = a.lmax;
   const int mb = mbase_of(L, m);
-  CH ch[LEG_K];
+  DfChain ch[LEG_K];
   float4 accE[LEG_K], accO[LEG_K];
 #pragma unroll
   for (int k = 0; k < LEG_K; ++k) {
@@ -512,7 +500,6 @@ __device__ __forceinline__ void df4_add(float4& a4, const float4 b4) {
 // warp reduces the slots over its 32 lanes through the transpose: lane t sums
 // one float pair (degree t / 4, re or im) over 16 lanes, and the two halves
 // are combined with one shuffle.
-template <class CH>
 __global__ void __launch_bounds__(128, 5) legendre_adj_df_k(LegArgs a, const double2* __restrict__ Gt,
                                                          float4* __restrict__ partial, int nitems, int64_t nalm) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -525,7 +512,7 @@ __global__ void __launch_bounds__(128, 5) legendre_adj_df_k(LegArgs a, const dou
   const int mb = mbase_of(L, m);
   const double sg = (m & 1) ? -1.0 : 1.0;
   const double2* row = Gt + (size_t)m * M;
-  CH ch[LEG_K];
+  DfChain ch[LEG_K];
   // folded spectrum per chain as double-float (hi_re, lo_re, hi_im, lo_im),
   // even / odd l - m, and the per-degree sums of each lane (rows padded to
   // 9 entries: conflict-free 16-byte stores)
@@ -569,11 +556,7 @@ __global__ void __launch_bounds__(128, 5) legendre_adj_df_k(LegArgs a, const dou
 #pragma unroll
     for (int k = 0; k < LEG_K; ++k) {
       if (ch[k].E == 0) {
-        float qh, ql;
-        qsplit(ch[k], qh, ql);
-        const float4 Sv = S[k * 128];
-        df_mac(acc.x, acc.y, Sv.x, Sv.y, qh, ql);
-        df_mac(acc.z, acc.w, Sv.z, Sv.w, qh, ql);
+        df_acc_step(acc, S[k * 128], ch[k]);
       }
     }
     *dst = acc;
@@ -986,14 +969,20 @@ static LegArgs make_args(nusht_plan_t p) {
 int legendre_build_tables(nusht_plan_t p, cudaStream_t s) {
   const int L = p->lmax, mmax = p->mmax, M = p->sz.M;
   const int64_t nalm = p->nalm;
-  std::vector<double> c(nalm), ah(nalm);
-  std::vector<int8_t> dsh(nalm, 0);
   // the double-float recurrence applies to the per-call kernels of mixed
   // plans and of FP64 plans with float-pair sums; it needs narrower segments
   const bool fastrec = p->opts.fast_recurrence && !(p->precision == NUSHT_FP64 && p->opts.fp64_contraction) &&
                        p->opts.legendre_table <= 0 && p->has_nufft;
+  // FP64 plans with float-pair sums run the two-degree recurrence
+  // (legendre2.cu) unless a recurrence table replaces it, and then need none
+  // of the one-degree tables
+  const bool two = p->precision == NUSHT_FP64 && !p->opts.fp64_contraction && p->has_nufft && !fastrec;
+  const bool one = !two || p->opts.legendre_table > 0;
+  const int64_t n1 = one ? nalm : 0;
+  std::vector<double> c(n1), ah(n1);
+  std::vector<int8_t> dsh(n1, 0);
   const int seg = fastrec ? LEG_SEG_BITS_DF : LEG_SEG_BITS;
-  for (int m = 0; m <= mmax; ++m) {
+  for (int m = 0; one && m <= mmax; ++m) {
     const int64_t mb = (int64_t)m * (2 * L + 1 - m) / 2;
     dd a2 = {1.0, 0.0};  // Ahat^2 (scaled)
     for (int l = m; l <= L; ++l) {
@@ -1044,13 +1033,18 @@ int legendre_build_tables(nusht_plan_t p, cudaStream_t s) {
   LegTables& t = p->leg;
   t.npairs = npairs;
   t.blocks_per_m = (npairs + LEG_PAIRS_PER_WARP - 1) / LEG_PAIRS_PER_WARP;
-  NUSHT_TRY(dev_alloc((void**)&t.c, nalm * 8, &p->bytes));
-  NUSHT_TRY(dev_alloc((void**)&t.ahat, nalm * 8, &p->bytes));
-  NUSHT_TRY(dev_alloc((void**)&t.dshift, nalm, &p->bytes));
   NUSHT_TRY(dev_alloc((void**)&t.cm, (mmax + 1) * 8, &p->bytes));
   NUSHT_TRY(dev_alloc((void**)&t.ring_x, npairs * 8, &p->bytes));
   NUSHT_TRY(dev_alloc((void**)&t.ring_s, npairs * 8, &p->bytes));
   NUSHT_TRY(dev_alloc((void**)&t.pole_norm, (L + 1) * 8, &p->bytes));
+  NUSHT_CUDA(cudaMemcpyAsync(t.cm, cm.data(), (mmax + 1) * 8, cudaMemcpyHostToDevice, s));
+  NUSHT_CUDA(cudaMemcpyAsync(t.ring_x, rx.data(), npairs * 8, cudaMemcpyHostToDevice, s));
+  NUSHT_CUDA(cudaMemcpyAsync(t.ring_s, rs.data(), npairs * 8, cudaMemcpyHostToDevice, s));
+  NUSHT_CUDA(cudaMemcpyAsync(t.pole_norm, pn.data(), (L + 1) * 8, cudaMemcpyHostToDevice, s));
+  if (!one) return leg2_setup(p, s);
+  NUSHT_TRY(dev_alloc((void**)&t.c, nalm * 8, &p->bytes));
+  NUSHT_TRY(dev_alloc((void**)&t.ahat, nalm * 8, &p->bytes));
+  NUSHT_TRY(dev_alloc((void**)&t.dshift, nalm, &p->bytes));
   NUSHT_CUDA(cudaMemcpyAsync(t.c, c.data(), nalm * 8, cudaMemcpyHostToDevice, s));
   if (fastrec) {
     std::vector<float2> cd(nalm);
@@ -1064,10 +1058,6 @@ int legendre_build_tables(nusht_plan_t p, cudaStream_t s) {
   }
   NUSHT_CUDA(cudaMemcpyAsync(t.ahat, ah.data(), nalm * 8, cudaMemcpyHostToDevice, s));
   NUSHT_CUDA(cudaMemcpyAsync(t.dshift, dsh.data(), nalm, cudaMemcpyHostToDevice, s));
-  NUSHT_CUDA(cudaMemcpyAsync(t.cm, cm.data(), (mmax + 1) * 8, cudaMemcpyHostToDevice, s));
-  NUSHT_CUDA(cudaMemcpyAsync(t.ring_x, rx.data(), npairs * 8, cudaMemcpyHostToDevice, s));
-  NUSHT_CUDA(cudaMemcpyAsync(t.ring_s, rs.data(), npairs * 8, cudaMemcpyHostToDevice, s));
-  NUSHT_CUDA(cudaMemcpyAsync(t.pole_norm, pn.data(), (L + 1) * 8, cudaMemcpyHostToDevice, s));
 
   // probe every (order, ring block), keep the significant ones (m ascending:
   // the longest recurrences are issued first)
@@ -1133,10 +1123,12 @@ int legendre_build_tables(nusht_plan_t p, cudaStream_t s) {
   }
 
   NUSHT_CUDA(cudaStreamSynchronize(s));
+  if (two && !t.tab) return leg2_setup(p, s);  // the table did not fit
   return NUSHT_OK;
 }
 
 int legendre_synth(nusht_plan_t p, const void* d_alm, cudaStream_t s) {
+  if (p->leg2.n2) return leg2_synth(p, d_alm, s);
   const int64_t nalm = p->nalm;
   const bool fastrec = p->leg.cdf != nullptr;  // opts.fast_recurrence (built when it applies)
   const int tb = 256;
@@ -1160,17 +1152,10 @@ int legendre_synth(nusht_plan_t p, const void* d_alm, cudaStream_t s) {
       poles_synth_k<float, float><<<1, 256, 0, s>>>((const float*)d_alm, p->leg.pole_norm, p->lmax, p->sz.M,
                                                     (float2*)p->G);
     }
-  } else if (p->precision == NUSHT_FP64 && !p->opts.fp64_contraction) {
+  } else if (p->precision == NUSHT_FP64 && !p->opts.fp64_contraction) {  // opts.fast_recurrence
     scale_alm_df_k<<<nb, tb, 0, s>>>((const double*)d_alm, p->leg.ahat, nalm, p->lmax, (float4*)p->atilde);
     if (nitems > 0)
-    {
-      if (fastrec)
-        legendre_synth_df_k<DfChain><<<(nitems + 3) / 4, 128, 0, s>>>(a, (const float4*)p->atilde, (double2*)p->G,
-                                                                      nitems);
-      else
-        legendre_synth_df_k<Chain><<<(nitems + 3) / 4, 128, 0, s>>>(a, (const float4*)p->atilde, (double2*)p->G,
-                                                                    nitems);
-    }
+      legendre_synth_df_k<<<(nitems + 3) / 4, 128, 0, s>>>(a, (const float4*)p->atilde, (double2*)p->G, nitems);
     poles_synth_k<double, double><<<1, 256, 0, s>>>((const double*)d_alm, p->leg.pole_norm, p->lmax, p->sz.M,
                                                     (double2*)p->G);
   } else if (p->precision == NUSHT_FP64) {
@@ -1198,6 +1183,7 @@ int legendre_synth(nusht_plan_t p, const void* d_alm, cudaStream_t s) {
 }
 
 int legendre_adjoint(nusht_plan_t p, void* d_alm, cudaStream_t s, double wpos) {
+  if (p->leg2.n2) return leg2_adjoint(p, d_alm, s, wpos);
   const int64_t nalm = p->nalm;
   const bool fastrec = p->leg.cdf != nullptr;
   LegArgs a = make_args(p);
@@ -1220,16 +1206,10 @@ int legendre_adjoint(nusht_plan_t p, void* d_alm, cudaStream_t s, double wpos) {
                                             p->leg.pole_norm, (const float2*)p->Ghat, p->lmax, p->sz.M, wpos,
                                             (float2*)d_alm);
     }
-  } else if (p->precision == NUSHT_FP64 && !p->opts.fp64_contraction) {
+  } else if (p->precision == NUSHT_FP64 && !p->opts.fp64_contraction) {  // opts.fast_recurrence
     if (nitems > 0)
-    {
-      if (fastrec)
-        legendre_adj_df_k<DfChain><<<(nitems + 3) / 4, 128, 0, s>>>(a, (const double2*)p->Ghat, (float4*)p->partial,
-                                                                    nitems, nalm);
-      else
-        legendre_adj_df_k<Chain><<<(nitems + 3) / 4, 128, 0, s>>>(a, (const double2*)p->Ghat, (float4*)p->partial,
-                                                                  nitems, nalm);
-    }
+      legendre_adj_df_k<<<(nitems + 3) / 4, 128, 0, s>>>(a, (const double2*)p->Ghat, (float4*)p->partial, nitems,
+                                                         nalm);
     adj_reduce_df_k<<<nb, tb, 0, s>>>((const float4*)p->partial, p->leg.blocks_per_m, nalm, p->leg.ahat,
                                       p->leg.pole_norm, (const double2*)p->Ghat, p->lmax, p->sz.M, wpos,
                                       (double2*)d_alm);

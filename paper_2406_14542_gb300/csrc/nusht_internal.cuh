@@ -81,6 +81,27 @@ struct LegTables {
   int npairs = 0;             // M/4
 };
 
+// The two-degree recurrence of FP64 plans (legendre2.cu); n2 entries, the
+// steps of every order one after another
+constexpr int LEG2_TINY_EXP = -74;         // smaller values are not summed
+constexpr int64_t LEG2_GROUPS_K1 = 12000;  // adjoint: fewer (order, 32-pair group) chains: one pair per lane
+constexpr int64_t LEG2_GROUPS_K2 = 40000;  // fewer: two, else four
+struct Leg2Tables {
+  int64_t n2 = 0;            // 0: the plan uses the one-degree kernels
+  double2* abx = nullptr;    // step factor coefficients for x^2 ...
+  double2* abs = nullptr;    // ... and for -sin^2
+  double* sc = nullptr;      // s_i
+  double* w1 = nullptr;      // s_i eps_{l_i}
+  double* w2 = nullptr;      // s_i eps_{l_i + 1}
+  int* gst = nullptr;        // first step per (order, group of 32 pairs)
+  int* ist = nullptr;        // first step per (order, pair)
+  double2* st = nullptr;     // the chain there
+  int* items_s = nullptr;    // work list of the synthesis: (order << 16) | group
+  int* items_a = nullptr;    // of the adjoint: (order << 16) | block of ka groups
+  int nis = 0, nia = 0;
+  int ka = 1;                // groups per block (pairs per lane) of the adjoint
+};
+
 struct PointData {
   int64_t npts = 0;
   int64_t cap = 0;
@@ -220,6 +241,7 @@ struct nusht_plan_s {
   int64_t nalm = 0;
 
   nusht::LegTables leg;
+  nusht::Leg2Tables leg2;
   nusht::PointData pts;
 
   // kernel Fourier factors: d1[k + lmax] (k = -lmax..lmax), d2[m] (m = 0..mmax)
@@ -304,6 +326,15 @@ int legendre_synth(nusht_plan_t p, const void* d_alm, cudaStream_t s);
 // wpos: factor of the m > 0 coefficients (1: the adjoint; 2: the gradient of a
 // real loss with respect to complex a_lm)
 int legendre_adjoint(nusht_plan_t p, void* d_alm, cudaStream_t s, double wpos = 1.0);
+
+// the two-degree recurrence (legendre2.cu): entries of its tables, set-up,
+// bytes of the adjoint's partial sums, execution
+int64_t leg2_entries(int lmax, int mmax);
+int leg2_setup(nusht_plan_t p, cudaStream_t s);
+size_t leg2_partial_bytes(nusht_plan_t p);
+void leg2_free(nusht_plan_t p);
+int leg2_synth(nusht_plan_t p, const void* d_alm, cudaStream_t s);
+int leg2_adjoint(nusht_plan_t p, void* d_alm, cudaStream_t s, double wpos);
 
 // NUFFT steps (nufft.cu)
 int deconv_pad(nusht_plan_t p, cudaStream_t s);

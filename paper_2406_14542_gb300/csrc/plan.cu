@@ -204,6 +204,7 @@ static void plan_free(nusht_plan_t p) {
   cudaSetDevice(p->device);
   free_points(p);
   spin_free(p);
+  leg2_free(p);
   dev_free(p->leg.c);
   dev_free(p->leg.cdf);
   dev_free(p->leg.ahat);
@@ -379,7 +380,9 @@ static int plan_body(nusht_plan_t p, int64_t npts, const double* d_pts, cudaStre
     NUSHT_CUDA(cudaStreamSynchronize(s));
   }
   if (role.legendre) {
-    NUSHT_TRY(dev_alloc(&p->atilde, (size_t)p->nalm * cplx, &p->bytes));
+    // nalm coefficients, or the two float4 per step of the two-degree
+    // recurrence: 2 ((lmax - m) / 2 + 1) <= lmax - m + 2 entries per order
+    NUSHT_TRY(dev_alloc(&p->atilde, (size_t)(p->nalm + z.mmax + 1) * cplx, &p->bytes));
     NUSHT_TRY(dev_alloc(&p->G, gbytes, &p->bytes));
     NUSHT_CUDA(cudaMemsetAsync(p->G, 0, gbytes, s));
   }
@@ -392,8 +395,12 @@ static int plan_body(nusht_plan_t p, int64_t npts, const double* d_pts, cudaStre
   NUSHT_TRY(dev_alloc(&p->fine, (size_t)z.n1 * (z.n2 / 2 + 1) * cplx, &p->bytes));
   if (role.legendre) {
     NUSHT_TRY(legendre_build_tables(p, s));
-    NUSHT_TRY(dev_alloc(&p->partial, (size_t)p->leg.blocks_per_m * p->nalm * cplx, &p->bytes));
-    NUSHT_CUDA(cudaMemsetAsync(p->partial, 0, (size_t)p->leg.blocks_per_m * p->nalm * cplx, s));
+    if (p->leg2.n2) {
+      NUSHT_TRY(dev_alloc(&p->partial, leg2_partial_bytes(p), &p->bytes));
+    } else {
+      NUSHT_TRY(dev_alloc(&p->partial, (size_t)p->leg.blocks_per_m * p->nalm * cplx, &p->bytes));
+      NUSHT_CUDA(cudaMemsetAsync(p->partial, 0, (size_t)p->leg.blocks_per_m * p->nalm * cplx, s));
+    }
     if (p->opts.spin > 0) NUSHT_TRY(spin_setup(p, s));
   }
   NUSHT_TRY(make_ffts(p, d1.data(), d2.data()));
