@@ -70,6 +70,26 @@ __device__ __forceinline__ void df_mac(float& sh, float& sl, float ah, float al,
   sl = __fsub_rn(l, __fsub_rn(sh, s));
 }
 
+// (h + l) = (ah + al) * (qh + ql), the low word not yet renormalised
+// (|l| < 2^-22 |h|): the first term of a short sum
+__device__ __forceinline__ void df_prod(float& h, float& l, float ah, float al, float qh, float ql) {
+  h = __fmul_rn(ah, qh);
+  l = __fmaf_rn(ah, ql, __fmaf_rn(al, qh, __fmaf_rn(ah, qh, -h)));
+}
+
+// df_mac without the renormalisation: the low word's rounding grows with the
+// number of terms, so only for sums of a few
+__device__ __forceinline__ void df_mac_open(float& sh, float& sl, float ah, float al, float qh, float ql) {
+  const float p = __fmul_rn(ah, qh);
+  const float e = __fmaf_rn(ah, qh, -p);
+  const float t = __fmaf_rn(ah, ql, __fmaf_rn(al, qh, e));
+  const float s = __fadd_rn(sh, p);
+  const float bp = __fsub_rn(s, sh);
+  const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bp)), __fsub_rn(p, bp));
+  sl = __fadd_rn(sl, __fadd_rn(err, t));
+  sh = s;
+}
+
 // (ah + al) += (bh + bl)
 __device__ __forceinline__ void df_add(float& ah, float& al, float bh, float bl) {
   const float s = __fadd_rn(ah, bh);

@@ -46,8 +46,11 @@
 
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 #include <vector>
 
+#include "async_copy.cuh"
+#include "ddouble.cuh"
 #include "dfloat.cuh"
 #include "nusht_internal.cuh"
 #include "recurrence.cuh"
@@ -88,60 +91,48 @@ __device__ __forceinline__ double step_arg(const Leg2Args& a, int j, bool pol) {
 // ---------------------------------------------------------------------------
 // plan time: recurrence tables (double-double) and chain starts
 // ---------------------------------------------------------------------------
-struct dd {
-  double hi, lo;
-};
-__device__ __forceinline__ dd dd_fast(double a, double b) {
-  const double s = a + b;
-  return {s, b - (s - a)};
-}
-__device__ __forceinline__ dd dd_mul(dd a, double b) {
-  const double p = a.hi * b;
-  return dd_fast(p, fma(a.lo, b, fma(a.hi, b, -p)));
-}
-__device__ __forceinline__ dd dd_div(dd a, double b) {
-  const double q = a.hi / b;
-  const double r = fma(-q, b, a.hi) + a.lo;
-  return dd_fast(q, r / b);
-}
-__device__ __forceinline__ dd dd_quot(double a, double b) { return dd_div({a, 0.0}, b); }
-__device__ __forceinline__ dd dd_add(dd a, dd b) {
-  const double s = a.hi + b.hi, bb = s - a.hi;
-  return dd_fast(s, ((a.hi - (s - bb)) + (b.hi - bb)) + (a.lo + b.lo));
-}
-__device__ __forceinline__ double dd_root(dd a) {
-  const double s = sqrt(a.hi);
-  return s + (fma(-s, s, a.hi) + a.lo) / (2.0 * s);
-}
-
-// One thread per order runs the scale recurrence s_{i+1}^2 = s_{i-1}^2
-// (eps_l eps_{l-1})^2 / (eps_{l+1} eps_{l+2})^2 in double-double; numerators
-// and denominators are exact integers below 2^53.
-__global__ void leg2_tab_k(int L, int mmax, double2* __restrict__ abx, double2* __restrict__ abs,
-                           double* __restrict__ sc, double* __restrict__ w1, double* __restrict__ w2) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per order.  The scales are a running product over every other step,
+//   s_{i+1}^2 = s_{i-1}^2 (eps_l eps_{l-1})^2 / (eps_{l+1} eps_{l+2})^2,
+// in double-double (numerators and denominators are exact integers below
+// 2^53): each lane forms the factor of its step, a scan of stride two over the
+// warp the products.
+__global__ void __launch_bounds__(128) leg2_tab_k(int L, int mmax, double2* __restrict__ abx,
+                                                  double2* __restrict__ abs, double* __restrict__ sc,
+                                                  double* __restrict__ w1, double* __restrict__ w2) {
+  const int lane = threadIdx.x & 31;
+  const int m = blockIdx.x * 4 + (threadIdx.x >> 5);
   if (m > mmax) return;
   const int n = steps_of(L, m);
   const int64_t b0 = base_of(L, m);
   const double m2 = (double)m * m;
   auto num = [&](int l) { return (double)l * l - m2; };
   auto den = [&](int l) { return 4.0 * (double)l * l - 1.0; };
-  // s_0 = 1 / eps_{m+1}: p_0 = Pbar_mm; s_1 is free
-  dd sp = {0.0, 0.0}, s = dd_quot(den(m + 1), num(m + 1));  // s_{i-1}^2, s_i^2
-  for (int i = 0; i < n; ++i) {
-    const int l = m + 1 + 2 * i;
+  // s_{i+1}^2 of the two steps before the chunk; s_0 = 1 / eps_{m+1} (p_0 = Pbar_mm), s_1 is free
+  dd c0 = {1.0, 0.0}, c1 = dd_quot(den(m + 1), num(m + 1));
+  for (int base = 0; base < n; base += 32) {
+    const int i = base + lane, l = m + 1 + 2 * i;
     const double n0 = num(l), n1 = num(l + 1), n2 = num(l + 2), d0 = den(l), d1 = den(l + 1), d2 = den(l + 2);
-    dd nx;
+    dd v;
     if (i == 0) {
-      nx = {s.hi * sqrt((n0 / d0) / (n2 / d2)), 0.0};
+      v = {c1.hi * sqrt((n0 / d0) / (n2 / d2)), 0.0};
     } else {
-      nx = dd_div(dd_div(dd_mul(dd_mul(sp, n0), num(l - 1)), n1), n2);
-      nx = dd_div(dd_div(dd_mul(dd_mul(nx, d1), d2), d0), den(l - 1));
+      v = dd_div(dd_div(dd_mul(dd_mul({n0, 0.0}, num(l - 1)), d1), n1), n2);
+      v = dd_div(dd_div(dd_mul(v, d2), d0), den(l - 1));
     }
+    for (int off = 2; off < 32; off *= 2) {
+      const dd u = dd_up(v, off);
+      if (lane >= off) v = dd_mul(v, u);
+    }
+    v = dd_mul(v, (lane & 1) ? c1 : c0);  // s_{i+1}^2
+    dd s = dd_up(v, 1);                   // s_i^2
+    if (lane == 0) s = c1;
+    c0 = {__shfl_sync(FULL, v.hi, 30), __shfl_sync(FULL, v.lo, 30)};
+    c1 = {__shfl_sync(FULL, v.hi, 31), __shfl_sync(FULL, v.lo, 31)};
+    if (i >= n) continue;
     // a_i^2 = s_i^2 / (eps_{l+1}^2 eps_{l+2}^2 s_{i+1}^2)
     dd a2 = dd_div(dd_div(dd_mul(dd_mul(s, d1), d2), n1), n2);
-    a2 = dd_div(a2, nx.hi);  // the last factor to first order in its low word
-    const double a = dd_root({a2.hi, a2.lo - a2.hi * (nx.lo / nx.hi)});
+    a2 = dd_div(a2, v.hi);  // the low word of the divisor to first order
+    const double a = dd_root({a2.hi, a2.lo - a2.hi * (v.lo / v.hi)});
     const dd e = dd_add(dd_quot(n0, d0), dd_quot(n1, d1));  // eps_l^2 + eps_{l+1}^2
     const dd bx = dd_mul(e, -a), bs = dd_mul(dd_add({1.0, 0.0}, {-e.hi, -e.lo}), a);
     abx[b0 + i] = make_double2(a, bx.hi + bx.lo);
@@ -149,8 +140,6 @@ __global__ void leg2_tab_k(int L, int mmax, double2* __restrict__ abx, double2* 
     sc[b0 + i] = dd_root(s);
     w1[b0 + i] = dd_root(dd_div(dd_mul(s, n0), d0));  // s_i eps_{l_i}
     w2[b0 + i] = dd_root(dd_div(dd_mul(s, n1), d1));  // s_i eps_{l_i + 1}
-    sp = s;
-    s = nx;
   }
 }
 
@@ -263,11 +252,10 @@ __global__ void __launch_bounds__(256) leg2_coef_k(const double2* __restrict__ a
 }
 
 // ---------------------------------------------------------------------------
-// synthesis: one 32-pair group per warp.  Two or four pairs per lane share the
-// coefficient loads but start at the earliest of their groups and leave fewer
-// warps: 21.2 / 22.9 ms against 21.3 at lmax 4095, 2.86 / 3.17 against 2.84 at
-// lmax 2047, 0.45 / 0.49 against 0.41 at lmax 1023.  At lmax 4095 the two
-// DFMAs per step take 18.9 ms of the FP64 pipe (the one-degree kernel: 52.0 ms).
+// synthesis: one 32-pair group per warp; two or four pairs per lane share the
+// coefficient reads but leave fewer warps and measured no faster at any size.
+// At lmax 4095 19.9 ms, of which the two DFMAs per step take 18.9 ms of the
+// FP64 pipe (the one-degree kernel: 52.0 ms).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) leg2_synth_k(Leg2Args a, const int* __restrict__ items, int nitems,
                                                     const float4* __restrict__ eo, double2* __restrict__ G) {
@@ -288,30 +276,46 @@ __global__ void __launch_bounds__(128) leg2_synth_k(Leg2Args a, const int* __res
   const int i0 = __ldg(a.gst + m * a.ngrp + g);
   double q1 = 0.0, q2 = 0.0;
   float4 E = make_float4(0.f, 0.f, 0.f, 0.f), O = E;
-  double2 ab = __ldg(tab + i0);
-  float4 ce = __ldg(ep + 2 * i0), co = __ldg(ep + 2 * i0 + 1);
-  for (int i = i0; i < n; ++i) {
-    // the next step's coefficients one step ahead (the last step reads its own again)
-    const int nx = min(i + 1, n - 1);
-    const double2 abn = __ldg(tab + nx);
-    const float4 cen = __ldg(ep + 2 * nx), con = __ldg(ep + 2 * nx + 1);
-    if (i == is) {
-      const double2 s = __ldg(a.st + so);
-      q1 = s.x;
-      q2 = s.y;
+  // the coefficients of 32 steps at a time through shared memory, the next 32
+  // in flight: a warp that has the SM to itself would otherwise wait for an L2
+  // read in every step (lmax 63: 10.8 -> 7.9 us; lmax 4095: 21.3 -> 19.9 ms)
+  __shared__ double2 s_ab[4][2][32];
+  __shared__ float4 s_eo[4][2][64];
+  double2(*ba)[32] = s_ab[threadIdx.x >> 5];
+  float4(*be)[64] = s_eo[threadIdx.x >> 5];
+  auto fetch = [&](int c, int buf) {
+    copy16(&ba[buf][lane], tab + min(c + lane, n - 1));
+    copy16(&be[buf][lane], ep + min(2 * c + lane, 2 * n - 1));
+    copy16(&be[buf][lane + 32], ep + min(2 * c + lane + 32, 2 * n - 1));
+  };
+  fetch(i0, 0);
+  copies_commit();
+  int buf = 0;
+  for (int c = i0; c < n; c += 32, buf ^= 1) {
+    if (c + 32 < n) fetch(c + 32, buf ^ 1);
+    copies_commit();
+    copies_wait<1>();
+    __syncwarp();
+    const int ns = min(32, n - c);
+    for (int t = 0; t < ns; ++t) {
+      const double2 ab = ba[buf][t];
+      const float4 ce = be[buf][2 * t], co = be[buf][2 * t + 1];
+      if (c + t == is) {
+        const double2 s = __ldg(a.st + so);
+        q1 = s.x;
+        q2 = s.y;
+      }
+      const double q = fma(fma(ab.x, z, ab.y), q1, -q2);
+      float qh, ql;
+      split_qr(q1, qh, ql);
+      q2 = q1;
+      q1 = q;
+      df_mac(E.x, E.y, ce.x, ce.y, qh, ql);
+      df_mac(E.z, E.w, ce.z, ce.w, qh, ql);
+      df_mac(O.x, O.y, co.x, co.y, qh, ql);
+      df_mac(O.z, O.w, co.z, co.w, qh, ql);
     }
-    const double q = fma(fma(ab.x, z, ab.y), q1, -q2);
-    float qh, ql;
-    split_qr(q1, qh, ql);
-    q2 = q1;
-    q1 = q;
-    df_mac(E.x, E.y, ce.x, ce.y, qh, ql);
-    df_mac(E.z, E.w, ce.z, ce.w, qh, ql);
-    df_mac(O.x, O.y, co.x, co.y, qh, ql);
-    df_mac(O.z, O.w, co.z, co.w, qh, ql);
-    ab = abn;
-    ce = cen;
-    co = con;
+    __syncwarp();  // the buffer is refilled by the next chunk
   }
   if (jn > a.npairs) return;
   // F(theta_j) = E + x O, F(pi - theta_j) = E - x O, doubled with (-1)^m
@@ -337,18 +341,24 @@ __global__ void __launch_bounds__(128) leg2_synth_k(Leg2Args a, const int* __res
 // shared-memory slots; every four steps the warp sums the slots over its 32
 // lanes through the transpose: lane t sums one float pair (slot t / 4, re or
 // im) over 16 lanes, one shuffle joins the halves.  K spreads that reduction
-// over more pairs but makes fewer warps (see leg2_setup): at lmax 4095
-// 28.7 / 24.5 / 23.2 ms with 1 / 2 / 4 pairs per lane (the one-degree kernel:
-// 52.6 ms), the FP64 pipe's share 18.9 ms.
+// over more pairs but makes fewer warps (see leg2_setup).  A lane's sums have
+// at most four terms, so they stay open (dfloat.cuh) until the transpose
+// renormalises them: 21.4 against 23.0 ms at lmax 4095, where the FP64 pipe's
+// share is 18.9 ms (the one-degree kernel: 52.6 ms).
 // ---------------------------------------------------------------------------
 template <int K>
-__global__ void __launch_bounds__(128) leg2_adj_k(Leg2Args a, const int* __restrict__ items, int nitems,
+__global__ void __launch_bounds__(128, 6) leg2_adj_k(Leg2Args a, const int* __restrict__ items, int nitems,
                                                   const double2* __restrict__ Gt, float4* __restrict__ partial,
                                                   int64_t n2) {
   // folded spectrum of the lane's chains, even and x odd, as float pairs; the
   // slots of a lane are padded to nine (conflict-free 16-byte stores)
   __shared__ float4 sS[2][K][128];
   __shared__ float4 red[4][32][9];
+  // step coefficients as in the synthesis; with four pairs per lane one step
+  // lasts 512 cycles and a read one step ahead is enough (22.9 against 23.4 ms
+  // at lmax 4095; with two pairs 566 against 546 us at lmax 1023)
+  constexpr bool STAGED = K < 4;
+  __shared__ double2 s_ab[STAGED ? 4 : 1][2][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int it = blockIdx.x * 4 + warp;
   if (it >= nitems) return;
@@ -395,17 +405,37 @@ __global__ void __launch_bounds__(128) leg2_adj_k(Leg2Args a, const int* __restr
   if (i0 >= n) return;
   float4* out = partial + (size_t)blk * 2 * n2 + 2 * b0;
   const int d = lane >> 2, cpt = (lane >> 1) & 1, half = lane & 1;
-  double2 ab = __ldg(tab + i0);
+  double2(*ba)[32] = s_ab[STAGED ? warp : 0];
+  auto fetch = [&](int c, int buf) {
+    copy16(&ba[buf][lane], tab + min(c + lane, n - 1));
+    copies_commit();
+  };
+  double2 ab = make_double2(0.0, 0.0);
+  if (STAGED)
+    fetch(i0, 0);
+  else
+    ab = __ldg(tab + i0);
   for (int base = i0; base < n; base += 4) {
+    const int at = base - i0, buf = (at >> 5) & 1;
+    if (STAGED && (at & 31) == 0) {
+      fetch(base + 32, buf ^ 1);
+      copies_wait<1>();
+      __syncwarp();
+    }
     const int ns = min(4, n - base);
 #pragma unroll 1
     for (int t = 0; t < ns; ++t) {
       const int i = base + t;
-      const double2 abn = __ldg(tab + min(i + 1, n - 1));
-      float4 e = make_float4(0.f, 0.f, 0.f, 0.f), o = e;
+      double2 abn = ab;
+      if (STAGED)
+        ab = ba[buf][(at & 31) + t];
+      else
+        abn = __ldg(tab + min(i + 1, n - 1));
+      float4 e, o;
+      // the group nearest the equator starts first: it opens the step's sums
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        if (K > 1 && i < gs[k]) continue;  // warp-uniform
+      for (int k = K - 1; k >= 0; --k) {
+        if (k < K - 1 && i < gs[k]) continue;  // warp-uniform
         if (i == is[k]) {
           const double2 s = __ldg(a.st + so + k * 32);
           q1[k] = s.x;
@@ -417,14 +447,21 @@ __global__ void __launch_bounds__(128) leg2_adj_k(Leg2Args a, const int* __restr
         q2[k] = q1[k];
         q1[k] = q;
         const float4 se = SE[k * 128], sd = SO[k * 128];
-        df_mac(e.x, e.y, se.x, se.y, qh, ql);
-        df_mac(e.z, e.w, se.z, se.w, qh, ql);
-        df_mac(o.x, o.y, sd.x, sd.y, qh, ql);
-        df_mac(o.z, o.w, sd.z, sd.w, qh, ql);
+        if (k == K - 1) {
+          df_prod(e.x, e.y, se.x, se.y, qh, ql);
+          df_prod(e.z, e.w, se.z, se.w, qh, ql);
+          df_prod(o.x, o.y, sd.x, sd.y, qh, ql);
+          df_prod(o.z, o.w, sd.z, sd.w, qh, ql);
+        } else {
+          df_mac_open(e.x, e.y, se.x, se.y, qh, ql);
+          df_mac_open(e.z, e.w, se.z, se.w, qh, ql);
+          df_mac_open(o.x, o.y, sd.x, sd.y, qh, ql);
+          df_mac_open(o.z, o.w, sd.z, sd.w, qh, ql);
+        }
       }
+      if (!STAGED) ab = abn;
       rw[lane][2 * t] = e;
       rw[lane][2 * t + 1] = o;
-      ab = abn;
     }
     __syncwarp();
     float sh = 0.f, sl = 0.f;
@@ -540,21 +577,36 @@ int leg2_setup(nusht_plan_t p, cudaStream_t s) {
   t.n2 = leg2_entries(L, mmax);
   const int ngrp = (p->leg.npairs + 31) / 32;
   // the adjoint's pairs per lane, by the number of (order, group) chains; with
-  // 1 / 2 / 4, kernel and partial reduction take 118 / 177 / 265 us at 2,700
-  // (lmax 517, mmax 301), 580 / 572 / 670 at 16,400 (lmax 1023), 3,990 / 3,450 /
-  // 3,290 at 65,500 (lmax 2047)
+  // 1 / 2 / 4, kernel and partial reduction take 104 / 131 / 240 us at 2,700
+  // (lmax 517, mmax 301), 471 / 463 / 624 at 16,400 (lmax 1023), 3,200 / 2,950 /
+  // 3,030 at 65,500 (lmax 2047), 23.8 / 21.7 / 21.7 ms at 262,000 (lmax 4095),
+  // where four also halve the partial rows (2.2 GB)
   const int64_t groups = (int64_t)(mmax + 1) * ngrp;
   t.ka = groups < LEG2_GROUPS_K1 ? 1 : groups < LEG2_GROUPS_K2 ? 2 : 4;
   const size_t n2 = (size_t)t.n2, np = (size_t)(mmax + 1) * ngrp * 32;
-  NUSHT_TRY(dev_alloc((void**)&t.abx, n2 * 16, &p->bytes));
-  NUSHT_TRY(dev_alloc((void**)&t.abs, n2 * 16, &p->bytes));
-  NUSHT_TRY(dev_alloc((void**)&t.sc, n2 * 8, &p->bytes));
-  NUSHT_TRY(dev_alloc((void**)&t.w1, n2 * 8, &p->bytes));
-  NUSHT_TRY(dev_alloc((void**)&t.w2, n2 * 8, &p->bytes));
-  NUSHT_TRY(dev_alloc((void**)&t.gst, (size_t)groups * 4, &p->bytes));
-  NUSHT_TRY(dev_alloc((void**)&t.ist, np * 4, &p->bytes));
-  NUSHT_TRY(dev_alloc((void**)&t.st, np * 16, &p->bytes));
-  leg2_tab_k<<<(mmax + 32) / 32, 32, 0, s>>>(L, mmax, t.abx, t.abs, t.sc, t.w1, t.w2);
+  // one allocation: at small lmax a plan costs what its allocations cost
+  char* at = nullptr;
+  auto carve = [&](auto*& q, size_t n) {
+    q = reinterpret_cast<std::remove_reference_t<decltype(q)>>(at);
+    at += (n * sizeof(*q) + 255) / 256 * 256;
+  };
+  auto layout = [&]() {
+    carve(t.abx, n2);
+    carve(t.abs, n2);
+    carve(t.st, np);
+    carve(t.sc, n2);
+    carve(t.w1, n2);
+    carve(t.w2, n2);
+    carve(t.ist, np);
+    carve(t.gst, (size_t)groups);
+    carve(t.items_s, (size_t)groups);
+    carve(t.items_a, (size_t)groups);
+  };
+  layout();
+  NUSHT_TRY(dev_alloc(&t.slab, (size_t)at, &p->bytes));
+  at = (char*)t.slab;
+  layout();
+  leg2_tab_k<<<(mmax + 4) / 4, 128, 0, s>>>(L, mmax, t.abx, t.abs, t.sc, t.w1, t.w2);
   leg2_start_k<<<(int)((groups + 3) / 4), 128, 0, s>>>(args_of(p), p->leg.cm, t.gst, t.ist, t.st);
   NUSHT_CUDA(cudaGetLastError());
   std::vector<int> gst((size_t)groups);
@@ -575,8 +627,6 @@ int leg2_setup(nusht_plan_t p, cudaStream_t s) {
   list(t.ka, ia);
   t.nis = (int)is.size();
   t.nia = (int)ia.size();
-  NUSHT_TRY(dev_alloc((void**)&t.items_s, std::max<size_t>(1, is.size()) * 4, &p->bytes));
-  NUSHT_TRY(dev_alloc((void**)&t.items_a, std::max<size_t>(1, ia.size()) * 4, &p->bytes));
   NUSHT_CUDA(cudaMemcpyAsync(t.items_s, is.data(), is.size() * 4, cudaMemcpyHostToDevice, s));
   NUSHT_CUDA(cudaMemcpyAsync(t.items_a, ia.data(), ia.size() * 4, cudaMemcpyHostToDevice, s));
   NUSHT_CUDA(cudaStreamSynchronize(s));
@@ -598,9 +648,7 @@ size_t leg2_partial_bytes(nusht_plan_t p) {
 
 void leg2_free(nusht_plan_t p) {
   Leg2Tables& t = p->leg2;
-  for (void* q : {(void*)t.abx, (void*)t.abs, (void*)t.sc, (void*)t.w1, (void*)t.w2, (void*)t.gst, (void*)t.ist,
-                  (void*)t.st, (void*)t.items_s, (void*)t.items_a})
-    dev_free(q);
+  dev_free(t.slab);
   t = Leg2Tables();
 }
 

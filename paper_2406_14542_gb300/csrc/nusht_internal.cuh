@@ -85,9 +85,10 @@ struct LegTables {
 // steps of every order one after another
 constexpr int LEG2_TINY_EXP = -74;         // smaller values are not summed
 constexpr int64_t LEG2_GROUPS_K1 = 12000;  // adjoint: fewer (order, 32-pair group) chains: one pair per lane
-constexpr int64_t LEG2_GROUPS_K2 = 40000;  // fewer: two, else four
+constexpr int64_t LEG2_GROUPS_K2 = 200000;  // fewer: two, else four
 struct Leg2Tables {
   int64_t n2 = 0;            // 0: the plan uses the one-degree kernels
+  void* slab = nullptr;      // holds every array below
   double2* abx = nullptr;    // step factor coefficients for x^2 ...
   double2* abs = nullptr;    // ... and for -sin^2
   double* sc = nullptr;      // s_i
