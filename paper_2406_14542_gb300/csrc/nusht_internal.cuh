@@ -210,20 +210,21 @@ struct NufftBatch {
 // two ring maps (Q and U; theta spectra in the adjoint) and the partial rows
 // of the adjoint
 struct SpinTables {
-  double* A = nullptr;        // sqrt((2l+1)(2l-1)) l / sqrt((l^2-m^2)(l^2-s^2))
-  double* Ab = nullptr;       // A m s / (l (l-1))
-  double* C = nullptr;        // the l-2 coefficient
-  double* st_mant = nullptr;  // start value at max(m, s) per (m, sign): mantissa ...
-  int* st_exp = nullptr;      // ... binary exponent ...
-  int* st_ab = nullptr;       // ... and powers of cos and sin of theta / 2 (a << 16 | b)
+  double2* abx = nullptr;     // step coefficients (a, b) for x, ...
+  double2* abs = nullptr;     // ... (a, a + b) for x - 1 ...
+  double* bmx = nullptr;      // ... and of the lambda- chain: -b, a - b
+  double* bms = nullptr;
+  double* sc = nullptr;       // scales s_l (0 below the first degree)
+  int* gst = nullptr;         // first degree per (order, group of 32 ring pairs)
+  int* ist = nullptr;         // first degree per (chain, order, pair)
+  double2* st = nullptr;      // the chain there
   double2* GQ = nullptr;      // [mmax + 1][M]
   double2* GU = nullptr;
-  float4* ap = nullptr;       // per call: (G + iC) / 2 and (-1)^s (G - iC) / 2 as float pairs
+  float4* ap = nullptr;       // per call: s_l (G + iC) / 2 and s_l (-1)^s (G - iC) / 2 as float pairs
   float4* am = nullptr;
   float4* pg = nullptr;       // [nrows][nalm] float-pair partial sums of G and C
   float4* pc = nullptr;
-  unsigned char* keep = nullptr;  // per (order, ring block): bit k = pass k has a value above 2^-300
-  int nrows = 0;
+  int nrows = 0;              // groups of 32 ring pairs
 };
 
 struct StageEvents {

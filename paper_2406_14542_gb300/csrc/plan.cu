@@ -607,7 +607,7 @@ int nusht_synth_grad_pts(nusht_plan_t p, const void* d_alm, const void* d_cot, d
 int nusht_synth_spin(nusht_plan_t p, const void* d_glm, const void* d_clm, void* d_q, void* d_u,
                      nusht_stream_t stream) {
   if (!p) return set_error(NUSHT_EINVAL, "plan is NULL");
-  if (p->opts.spin <= 0 || !p->spin.A) return set_error(NUSHT_EUNSUPPORTED, "plan made without opts.spin");
+  if (p->opts.spin <= 0 || !p->spin.abx) return set_error(NUSHT_EUNSUPPORTED, "plan made without opts.spin");
   if (!d_glm || !d_clm || (p->pts.npts > 0 && (!d_q || !d_u))) return set_error(NUSHT_EINVAL, "null pointer");
   cudaStream_t s = (cudaStream_t)stream;
   // S for both fields at once (the Wigner-d recurrences are shared), then
@@ -625,7 +625,7 @@ int nusht_synth_spin(nusht_plan_t p, const void* d_glm, const void* d_clm, void*
 int nusht_adjoint_spin(nusht_plan_t p, const void* d_q, const void* d_u, void* d_glm, void* d_clm,
                        nusht_stream_t stream) {
   if (!p) return set_error(NUSHT_EINVAL, "plan is NULL");
-  if (p->opts.spin <= 0 || !p->spin.A) return set_error(NUSHT_EUNSUPPORTED, "plan made without opts.spin");
+  if (p->opts.spin <= 0 || !p->spin.abx) return set_error(NUSHT_EUNSUPPORTED, "plan made without opts.spin");
   if (!d_glm || !d_clm || (p->pts.npts > 0 && (!d_q || !d_u))) return set_error(NUSHT_EINVAL, "null pointer");
   cudaStream_t s = (cudaStream_t)stream;
   // N^dagger and F^dagger for each field into its theta-spectrum buffer, then
