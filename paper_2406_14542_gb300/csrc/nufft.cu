@@ -23,6 +23,7 @@
 
 #include "nusht_internal.cuh"
 #include "dfloat.cuh"
+#include "tc_pack.cuh"
 
 namespace nusht {
 
@@ -106,11 +107,12 @@ __global__ void prep_k(const double* __restrict__ pts, int64_t npts, int n1, int
 }
 
 // sorted point s <- caller's point perm[s]: first taps, and kernel values
-// (FP64: psi[s][0..w) along theta then psi[s][w..2w) along phi) or the
+// (FP64: psi[s][0..w) along theta then psi[s][w..2w) along phi; psid as float
+// pairs, with `packed` those along phi as packed digits, tc_pack.cuh) or the
 // offsets (MIXED, kernel evaluated on the fly in float)
 __global__ void gather_k(const double* __restrict__ pts, const int* __restrict__ perm, int64_t npts, int n1, int n2,
                          int w, double beta, int* __restrict__ cell, double* __restrict__ psi,
-                         float2* __restrict__ psid, float* __restrict__ offf, double* __restrict__ xy) {
+                         float2* __restrict__ psid, bool packed, float* __restrict__ offf, double* __restrict__ xy) {
   int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= npts) return;
   const int i = perm[s];
@@ -138,6 +140,10 @@ __global__ void gather_k(const double* __restrict__ pts, const int* __restrict__
     }
     for (int b = 0; b < w; ++b) {
       const double v = es_psi((o2 - b) * sc, beta);
+      if (packed) {
+        reinterpret_cast<uint2*>(ps)[w + b] = tc_pack(v);
+        continue;
+      }
       const float h = __double2float_rn(v);
       ps[w + b] = make_float2(h, __double2float_rn(v - (double)h));
     }
@@ -588,7 +594,8 @@ __global__ void __launch_bounds__(IDF_THREADS) interp_grad_df_k(const double* __
                                                                 const int* __restrict__ cell,
                                                                 const float2* __restrict__ psi,
                                                                 const double* __restrict__ xy,
-                                                                const int* __restrict__ perm, float2 beta,
+                                                                const int* __restrict__ perm, bool packed,
+                                                                float2 beta,
                                                                 double* __restrict__ dth, double* __restrict__ dph,
                                                                 double* __restrict__ ptg,
                                                                 const double* __restrict__ cot,
@@ -620,7 +627,7 @@ __global__ void __launch_bounds__(IDF_THREADS) interp_grad_df_k(const double* __
     float2 p2[W], q2[W];
 #pragma unroll
     for (int b = 0; b < W; ++b) {
-      p2[b] = ps[W + b];
+      p2[b] = packed ? tc_value(reinterpret_cast<const uint2*>(ps)[W + b]) : ps[W + b];
       q2[b] = df_mul(p2[b], es_dfac<W>(o2h, o2l, b, beta));
     }
     float th = 0.f, tl = 0.f, fh = 0.f, fl = 0.f;
@@ -784,10 +791,10 @@ void launch_interp_df(int nsub, size_t sm, cudaStream_t s, const double* grid, i
 template <int W>
 void launch_interp_grad_df(int nsub, size_t sm, cudaStream_t s, const double* grid, int64_t stride, int n1, int n2,
                            int nb2, int binsz, const int* sub, const int* cell, const float2* psi, const double* xy,
-                           const int* perm, float2 beta, double* dth, double* dph, double* ptg, const double* cot,
-                           double* gpts) {
-  interp_grad_df_k<W><<<nsub, IDF_THREADS, sm, s>>>(grid, stride, n1, n2, nb2, binsz, sub, cell, psi, xy, perm, beta,
-                                                    dth, dph, ptg, cot, gpts);
+                           const int* perm, bool packed, float2 beta, double* dth, double* dph, double* ptg,
+                           const double* cot, double* gpts) {
+  interp_grad_df_k<W><<<nsub, IDF_THREADS, sm, s>>>(grid, stride, n1, n2, nb2, binsz, sub, cell, psi, xy, perm,
+                                                    packed, beta, dth, dph, ptg, cot, gpts);
 }
 
 template <int W>
@@ -1172,7 +1179,7 @@ int spread_smem_optin() {
     NUSHT_W_DISPATCH(w, optin_f, &bad);
   }
   if (bad) return set_error(NUSHT_ECUDA, "shared-memory opt-in for the double-float NUFFT kernels");
-  return NUSHT_OK;
+  return tc_smem_optin();
 }
 
 void free_points(nusht_plan_t p) {
@@ -1409,7 +1416,7 @@ int setpts_impl(nusht_plan_t p, int64_t npts, const double* d_pts, cudaStream_t 
   const bool dfm = nufft_df(p);
   gather_k<<<nblk, tb, 0, s>>>(d_pts, d.perm, npts, z.n1, z.n2, z.w, z.beta, d.cell,
                                dbl && !dfm ? d.psi : nullptr, dfm ? reinterpret_cast<float2*>(d.psi) : nullptr,
-                               dbl ? nullptr : d.off, d.xy);
+                               nufft_tc(p), dbl ? nullptr : d.off, d.xy);
   NUSHT_CUDA(cudaGetLastError());
   NUSHT_CUDA(cudaStreamSynchronize(s));
   return NUSHT_OK;
@@ -1460,6 +1467,7 @@ int interp(nusht_plan_t p, void* d_map, cudaStream_t s) {
   const int nb = (int)((n + tb - 1) / tb);
   if (nufft_df(p)) {
     if (p->pts.nsub == 0) return NUSHT_OK;
+    if (nufft_tc(p)) return tc_interp(p, (double*)d_map, s);
     const int binsz = p->pts.bin > 0 ? p->pts.bin : 32;
     const int tw = binsz + z.w - 1;
     NUSHT_W_DISPATCH(z.w, launch_interp_df, p->pts.nsub, (size_t)tw * tw * 8, s, (const double*)p->fine, stride,
@@ -1488,8 +1496,8 @@ static int interp_grad_df(nusht_plan_t p, double* d_dth, double* d_dph, double* 
   const float2 beta = make_float2(bh, (float)(z.beta - (double)bh));
   NUSHT_W_DISPATCH(z.w, launch_interp_grad_df, p->pts.nsub, (size_t)tw * tw * 8, s, (const double*)p->fine, stride,
                    z.n1, z.n2, p->pts.nbins2, binsz, p->pts.sub, p->pts.cell,
-                   reinterpret_cast<const float2*>(p->pts.psi), p->pts.xy, p->pts.perm, beta, d_dth, d_dph, d_ptg,
-                   cot, gpts);
+                   reinterpret_cast<const float2*>(p->pts.psi), p->pts.xy, p->pts.perm, nufft_tc(p), beta, d_dth,
+                   d_dph, d_ptg, cot, gpts);
   NUSHT_CUDA(cudaGetLastError());
   return NUSHT_OK;
 }
@@ -1546,7 +1554,9 @@ int spread(nusht_plan_t p, const void* d_map, cudaStream_t s) {
   const int tw = binsz + z.w - 1;
   // FP32 spreading kernels stage the subproblem's points after the tile
   const size_t sm = p->precision == NUSHT_FP64 ? (size_t)tw * tw * es : spread_f_smem(tw);
-  if (nufft_df(p)) {
+  if (nufft_tc(p)) {
+    NUSHT_TRY(tc_spread(p, (const double*)d_map, det ? (float2*)p->pts.tiles : nullptr, s));
+  } else if (nufft_df(p)) {
     const size_t smd = (size_t)tw * spread_df_stride(tw, z.w) * 8 + (size_t)SUBMAX * 16;
     NUSHT_W_DISPATCH(z.w, launch_spread_df, p->pts.nsub, smd, s, (double*)p->fine, stride, z.n1,
                      z.n2, p->pts.nbins2, binsz, p->pts.sub, p->pts.cell,

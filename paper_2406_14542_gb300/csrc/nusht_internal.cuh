@@ -348,6 +348,14 @@ int interp_grad(nusht_plan_t p, void* d_dth, void* d_dph, const void* cot, doubl
 int interp_pointing(nusht_plan_t p, double* d_ptg, cudaStream_t s);
 int spread(nusht_plan_t p, const void* d_map, cudaStream_t s);
 int spread_smem_optin();
+// the same on the tensor cores (nufft_tc.cu): whether a plan's point set takes
+// that path, shared-memory opt-in, execution (tiles: deterministic mode)
+constexpr int TC_WMIN = 12;  // narrower kernels: float pairs
+constexpr int TC_FILL = 16;  // fewer points per subproblem on average: float pairs
+bool nufft_tc(nusht_plan_t p);
+int tc_smem_optin();
+int tc_interp(nusht_plan_t p, double* d_map, cudaStream_t s);
+int tc_spread(nusht_plan_t p, const double* d_map, float2* tiles, cudaStream_t s);
 // every member of a NufftBatch (mixed precision, atomics): zero the fine
 // grids, spread the maps (caller order, maps[i] of member i), interpolate
 int zero_grids_many(const NufftBatch& nb, cudaStream_t s);
