@@ -62,11 +62,6 @@ namespace {
 using namespace rec;
 constexpr unsigned FULL = 0xffffffffu;
 
-// entries of order m: n = (L - m) / 2 + 1 steps; first entry of order m
-__host__ __device__ __forceinline__ int steps_of(int L, int m) { return (L - m) / 2 + 1; }
-__host__ __device__ __forceinline__ int64_t tri2(int64_t k) { return k * k / 4 + k + 1; }  // sum_{j<=k} (j / 2 + 1)
-__host__ __device__ __forceinline__ int64_t base_of(int L, int m) { return tri2(L) - tri2((int64_t)L - m); }
-
 struct Leg2Args {
   int lmax, mmax, M, npairs, ngrp, kblk;
   const double2* abx;  // (a_i, b_i): step factor a x^2 + b

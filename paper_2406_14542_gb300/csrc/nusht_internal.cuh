@@ -74,7 +74,7 @@ struct LegTables {
   int nitems = 0;
   int nitems_total = 0;
   int64_t triples = 0;        // (ring pair, l, m) triples of the kept items
-  void* tab = nullptr;        // recurrence table (table mode): float or float2 per triple
+  void* tab = nullptr;        // recurrence table of FP64 plans (table mode): float2 per triple
   int64_t* tab_off = nullptr; // per-item offsets into tab
   size_t tab_bytes = 0;
   int blocks_per_m = 0;       // ring blocks per order
@@ -101,6 +101,24 @@ struct Leg2Tables {
   int* items_a = nullptr;    // of the adjoint: (order << 16) | block of ka groups
   int nis = 0, nia = 0;
   int ka = 1;                // groups per block (pairs per lane) of the adjoint
+};
+
+// The recurrence table of mixed plans (legtab.cu); steps as in legendre2.cu
+constexpr double TAB_XMIN = 0.25;  // cos(theta) down to which the adjoint reads the odd degrees only
+struct LegTab {
+  float4* tab = nullptr;   // null: the plan has none
+  void* slab = nullptr;    // holds every array below
+  int64_t* off = nullptr;  // first chunk per (order, group of 32 ring pairs)
+  int* gst = nullptr;      // first step per (order, group)
+  double* sc = nullptr;    // Ahat_l of the odd degrees l, ...
+  double* w1 = nullptr;    // ... times eps_l ...
+  double* w2 = nullptr;    // ... and times eps_{l + 1}
+  float4* ao = nullptr;    // per call: scaled coefficients of a step's two degrees
+  int* items_s = nullptr;  // work lists: (order << 16) | group, block of four groups
+  int* items_a = nullptr;
+  int nis = 0, nia = 0;
+  int nA = 0;              // blocks (from the pole) whose odd degrees serve both parities
+  int64_t n2 = 0;
 };
 
 struct PointData {
@@ -244,6 +262,7 @@ struct nusht_plan_s {
 
   nusht::LegTables leg;
   nusht::Leg2Tables leg2;
+  nusht::LegTab tab;
   nusht::PointData pts;
 
   // kernel Fourier factors: d1[k + lmax] (k = -lmax..lmax), d2[m] (m = 0..mmax)
@@ -337,6 +356,18 @@ size_t leg2_partial_bytes(nusht_plan_t p);
 void leg2_free(nusht_plan_t p);
 int leg2_synth(nusht_plan_t p, const void* d_alm, cudaStream_t s);
 int leg2_adjoint(nusht_plan_t p, void* d_alm, cudaStream_t s, double wpos);
+// index of the steps: n = (lmax - m) / 2 + 1 of order m, and its first entry
+__host__ __device__ __forceinline__ int steps_of(int L, int m) { return (L - m) / 2 + 1; }
+__host__ __device__ __forceinline__ int64_t tri2(int64_t k) { return k * k / 4 + k + 1; }  // sum_{j<=k} (j / 2 + 1)
+__host__ __device__ __forceinline__ int64_t base_of(int L, int m) { return tri2(L) - tri2((int64_t)L - m); }
+
+// the recurrence table of mixed plans (legtab.cu): built where it fits in half
+// the free memory (p->tab.tab stays null otherwise), execution
+int legtab_setup(nusht_plan_t p, cudaStream_t s);
+void legtab_free(nusht_plan_t p);
+size_t legtab_partial_bytes(nusht_plan_t p);
+int legtab_synth(nusht_plan_t p, const void* d_alm, cudaStream_t s);
+int legtab_adjoint(nusht_plan_t p, void* d_alm, cudaStream_t s, double wpos);
 
 // NUFFT steps (nufft.cu)
 int deconv_pad(nusht_plan_t p, cudaStream_t s);

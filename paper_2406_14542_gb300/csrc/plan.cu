@@ -205,6 +205,7 @@ static void plan_free(nusht_plan_t p) {
   free_points(p);
   spin_free(p);
   leg2_free(p);
+  legtab_free(p);
   dev_free(p->leg.c);
   dev_free(p->leg.cdf);
   dev_free(p->leg.ahat);
@@ -395,8 +396,8 @@ static int plan_body(nusht_plan_t p, int64_t npts, const double* d_pts, cudaStre
   NUSHT_TRY(dev_alloc(&p->fine, (size_t)z.n1 * (z.n2 / 2 + 1) * cplx, &p->bytes));
   if (role.legendre) {
     NUSHT_TRY(legendre_build_tables(p, s));
-    if (p->leg2.n2) {
-      NUSHT_TRY(dev_alloc(&p->partial, leg2_partial_bytes(p), &p->bytes));
+    if (p->leg2.n2 || p->tab.tab) {
+      NUSHT_TRY(dev_alloc(&p->partial, p->tab.tab ? legtab_partial_bytes(p) : leg2_partial_bytes(p), &p->bytes));
     } else {
       NUSHT_TRY(dev_alloc(&p->partial, (size_t)p->leg.blocks_per_m * p->nalm * cplx, &p->bytes));
       NUSHT_CUDA(cudaMemsetAsync(p->partial, 0, (size_t)p->leg.blocks_per_m * p->nalm * cplx, s));
