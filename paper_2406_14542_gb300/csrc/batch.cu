@@ -2731,6 +2731,7 @@ int build_fused(nusht_batch_t p) {
     sub += q->pts.nsub;
     zero += (int)((z.n1 * a.stride + ZERO_CHUNK - 1) / ZERO_CHUNK);
     g.bin = std::max(g.bin, a.bin);
+    if (a.spread_rows) g.nsub_scattered += q->pts.nsub;
     if (p->fused_sfft) {
       SfftMember& f = sm[t];
       sfft_member(q, f);

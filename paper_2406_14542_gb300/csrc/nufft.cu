@@ -949,6 +949,113 @@ __global__ void __launch_bounds__(128) spread_pt_k(float* __restrict__ grid, int
   }
 }
 
+// Spreading in float by one warp per subproblem (6 <= w <= 8): the lanes take
+// the footprint of one point after the other, 8 columns x 4 rows, rows r and
+// r + 4, and add to the tile with plain loads and stores -- the lanes' cells
+// are distinct, so no atomics.  The kernel values of 32 points are evaluated
+// one point per lane, as in spread_point_f, and passed on through shared
+// memory.  A tile row is a multiple of 32 words + 8, so the 32 cells of a step
+// always lie in 32 banks.  Taps beyond w have weight 0 and stay inside the tile's padding.
+// What bounds it is the shared-memory pipe and issue: two loads and two stores
+// of the tile and two 8-byte loads of weights per point, the same for every w.
+// 32 uniform sets of lmax 256 to 1535, w 7, 60M points: 4.33 -> 2.82 ms.
+constexpr int SW_PT = 28;  // words per staged point: 4 (p1, p1') and 8 (p2, cell) pairs, padded
+constexpr int SW_WMIN = 6, SW_WMAX = 8;
+__host__ __device__ inline int sw_stride(int binsz) { return (binsz + 30) / 32 * 32 + 8; }
+inline size_t spread_warp_smem(int binsz) { return (size_t)(32 * SW_PT + (binsz + 7) * sw_stride(binsz)) * 4; }
+
+template <int W>
+__device__ __forceinline__ void spread_warp_sub(float* __restrict__ grid, int64_t stride, int n1, int n2, int r0,
+                                                int c0, int binsz, float beta, const int2* __restrict__ cell,
+                                                const float2* __restrict__ off, const int* __restrict__ perm,
+                                                const float* __restrict__ f, int start, int cnt, float* smem) {
+  static_assert(W >= SW_WMIN && W <= SW_WMAX, "");
+  const int lane = threadIdx.x & 31;
+  const int ts = sw_stride(binsz), tw = binsz + W - 1;
+  float* tile = smem + 32 * SW_PT;
+  for (int t = 4 * lane; t < (binsz + 7) * ts; t += 128) *(float4*)(tile + t) = make_float4(0.f, 0.f, 0.f, 0.f);
+  cell += start;
+  off += start;
+  perm += start;
+  const int r = lane >> 3, c = lane & 7;
+  float* my = tile + r * ts + c;
+  const float* wr = smem + 2 * r;
+  const float* wc = smem + 8 + 2 * c;
+  const float scf = 2.0f / W;
+  // one step ahead: the points' data, two steps ahead: their map index
+  int2 ce = make_int2(r0, c0);
+  float2 o = make_float2(0.f, 0.f);
+  float fv = 0.f;
+  if (lane < cnt) {
+    ce = cell[lane];
+    o = off[lane];
+    fv = f[perm[lane]];
+  }
+  int pm = lane + 32 < cnt ? perm[lane + 32] : 0;
+  for (int k0 = 0; k0 < cnt; k0 += 32) {
+    const bool on = k0 + lane < cnt;
+    float p1[8], p2[8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      p1[a] = a < W && on ? fv * es_psif((o.x - a) * scf, beta) : 0.f;
+      p2[a] = a < W && on ? es_psif((o.y - a) * scf, beta) : 0.f;
+    }
+    const float base = __int_as_float(on ? (ce.x - r0) * ts + (ce.y - c0) : 0);
+    float4* q = (float4*)(smem + lane * SW_PT);
+    q[0] = make_float4(p1[0], p1[4], p1[1], p1[5]);
+    q[1] = make_float4(p1[2], p1[6], p1[3], p1[7]);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) q[2 + a] = make_float4(p2[2 * a], base, p2[2 * a + 1], base);
+    __syncwarp();
+    if (k0 + 32 + lane < cnt) {
+      ce = cell[k0 + 32 + lane];
+      o = off[k0 + 32 + lane];
+      fv = f[pm];
+    }
+    if (k0 + 64 + lane < cnt) pm = perm[k0 + 64 + lane];
+    const int n = cnt - k0 < 32 ? cnt - k0 : 32;
+    for (int j = 0; j < n; j += 4) {  // points past the last one add zeros
+      float2 u[4], v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        u[i] = *(const float2*)(wr + (j + i) * SW_PT);
+        v[i] = *(const float2*)(wc + (j + i) * SW_PT);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float* t = my + __float_as_int(v[i].y);
+        const float x = t[0], y = t[4 * ts];
+        t[0] = fmaf(u[i].x, v[i].x, x);
+        t[4 * ts] = fmaf(u[i].y, v[i].x, y);
+        __syncwarp();
+      }
+    }
+  }
+  __syncwarp();
+  const float itw = 1.0f / (float)tw;  // exact row of t, as in spread_pt_k
+  for (int t = lane; t < tw * tw; t += 32) {
+    const int tr = __float2int_rz(((float)t + 0.5f) * itw), tc = t - tr * tw;
+    const float v = tile[tr * ts + tc];
+    if (v != 0.f) {
+      int rr = r0 + tr, cc = c0 + tc;
+      while (rr >= n1) rr -= n1;
+      while (cc >= n2) cc -= n2;
+      atomicAdd(grid + (int64_t)rr * stride + cc, v);
+    }
+  }
+}
+
+template <int W>
+__global__ void __launch_bounds__(32) spread_warp_k(float* __restrict__ grid, int64_t stride, int n1, int n2, int nb2,
+                                                    int binsz, float betaf, const int* __restrict__ sub,
+                                                    const int* __restrict__ cell, const float* __restrict__ offf,
+                                                    const int* __restrict__ perm, const float* __restrict__ f) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int bin = sub[3 * blockIdx.x], start = sub[3 * blockIdx.x + 1], cnt = sub[3 * blockIdx.x + 2];
+  spread_warp_sub<W>(grid, stride, n1, n2, (bin / nb2) * binsz, (bin % nb2) * binsz, binsz, betaf, (const int2*)cell,
+                     (const float2*)offf, perm, f, start, cnt, reinterpret_cast<float*>(smem_raw));
+}
+
 // interpolation in float (mixed mode): one thread per point, kernel values
 // evaluated on the fly from the FP32 offsets
 template <int W>
@@ -986,10 +1093,29 @@ __global__ void __launch_bounds__(128) interp_f_k(const float* __restrict__ grid
   out[perm[s]] = acc;
 }
 
+// Float spreading by spread_warp_k or by spread_pt_k (kernel times in us, the
+// latter first).  Scattered points (spread_rows), 2.09M uniform ones at lmax
+// 1023: w 5 91 / 107, w 6 120 / 112, w 7 153 / 111, w 8 193 / 116; on a ring
+// grid neighbours do not collide and the thread per point is as fast (w 7: 100
+// / 109).  One warp walks the up to 256 points of a subproblem, about 25 us,
+// which a few hundred subproblems do not hide (130,000 points at lmax 255: 19 /
+// 28); 500,000 points in about 2,000 of them: 54 / 32.
+constexpr int SW_NSUB = 2048;
+inline bool spread_by_warp(int w, int nsub, bool scattered) {
+  return w >= SW_WMIN && w <= SW_WMAX && scattered && nsub >= SW_NSUB;
+}
+
 template <int W>
 void launch_spread_f(int nsub, size_t sm, cudaStream_t s, float* grid, int64_t stride, int n1, int n2, int nb2,
                      int binsz, float betaf, const int* sub, const int* cell, const float* offf, const int* perm,
                      const float* f, int rows) {
+  if constexpr (W >= SW_WMIN && W <= SW_WMAX) {
+    if (spread_by_warp(W, nsub, rows != 0)) {
+      spread_warp_k<W><<<nsub, 32, spread_warp_smem(binsz), s>>>(grid, stride, n1, n2, nb2, binsz, betaf, sub, cell,
+                                                                 offf, perm, f);
+      return;
+    }
+  }
   spread_pt_k<W><<<nsub, 128, sm, s>>>(grid, stride, n1, n2, nb2, binsz, betaf, sub, cell, offf, perm, f, rows);
 }
 
@@ -1096,6 +1222,19 @@ __global__ void __launch_bounds__(128) spread_many_k(const NufftMember* __restri
 }
 
 template <int W>
+__global__ void __launch_bounds__(32) spread_warp_many_k(const NufftMember* __restrict__ mem, int nm, int base,
+                                                         const float* const* __restrict__ maps) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int b = blockIdx.x + base;
+  const int i = nufft_member_of<MEMBER_SUB>(mem, nm, b);
+  const NufftMember& q = mem[i];
+  const int* sb = q.sub + 3 * (b - q.sub0);
+  spread_warp_sub<W>(q.grid, q.stride, q.n1, q.n2, (sb[0] / q.nbins2) * q.bin, (sb[0] % q.nbins2) * q.bin, q.bin,
+                     q.beta, (const int2*)q.cell, (const float2*)q.off, q.perm, maps[i], sb[1], sb[2],
+                     reinterpret_cast<float*>(smem_raw));
+}
+
+template <int W>
 __global__ void __launch_bounds__(128) interp_many_k(const NufftMember* __restrict__ mem, int nm, int base,
                                                      float* const* __restrict__ maps) {
   const int b = blockIdx.x + base;
@@ -1151,6 +1290,12 @@ __global__ void deconv_trunc_many_k(const NufftMember* __restrict__ mem, int nm)
 
 template <int W>
 void launch_spread_many(const NufftBatch& nb, size_t sm, cudaStream_t s, const float* const* maps) {
+  if constexpr (W >= SW_WMIN && W <= SW_WMAX) {
+    if (spread_by_warp(W, nb.nsub, 2 * nb.nsub_scattered > nb.nsub)) {
+      spread_warp_many_k<W><<<nb.nsub, 32, spread_warp_smem(nb.bin), s>>>(nb.mem, nb.nm, nb.sub_base, maps);
+      return;
+    }
+  }
   spread_many_k<W><<<nb.nsub, 128, sm, s>>>(nb.mem, nb.nm, nb.sub_base, maps);
 }
 template <int W>

@@ -221,6 +221,7 @@ struct NufftBatch {
   int npad = 0, ntrunc = 0;          // blocks of the deconvolution launches
   int map_base = 0;                  // position of the slice in the batch's tables
   int bin = 32;                      // largest bin edge (spreading tile size)
+  int nsub_scattered = 0;            // subproblems of members with spread_rows
 };
 
 // Spin-weighted transforms (spin.cu): Wigner-d recurrence tables of the
