@@ -55,12 +55,15 @@ __device__ __forceinline__ double es_psi(double z, double beta) {
   double r = 1.0 - z * z;
   return r > 0.0 ? exp(beta * (sqrt(r) - 1.0)) : 0.0;
 }
-// exp(beta (sqrt(1 - z^2) - 1)) as 2^(beta log2(e) (sqrt(1 - z^2) - 1)): exp2f
-// is the shorter of the two on the GPU; spreading and interpolation share it,
-// so the FP32 adjoint stays the exact transpose
+// exp(beta (sqrt(1 - z^2) - 1)) as 2^(beta log2(e) (sqrt(1 - z^2) - 1)), by the
+// base-2 exponential instruction (at most 2 ulp, as exp2f; exp2f also serves
+// results below 2^-126, and beta < 64 keeps psi above 2^-93).  Spreading and
+// interpolation share it, so the FP32 adjoint stays the exact transpose.
 __device__ __forceinline__ float es_psif(float z, float beta) {
-  float r = 1.0f - z * z;
-  return r > 0.0f ? exp2f((beta * 1.44269504088896341f) * (sqrtf(r) - 1.0f)) : 0.0f;
+  const float r = 1.0f - z * z;
+  float v;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(v) : "f"((beta * 1.44269504088896341f) * (sqrtf(r) - 1.0f)));
+  return r > 0.0f ? v : 0.0f;
 }
 // d psi / dz
 __device__ __forceinline__ double es_dpsi(double z, double beta) {
