@@ -40,8 +40,12 @@
  *                contraction (sum_l a_lm P_lm and its adjoint), the theta FFT
  *                and the fine-grid 2D FFT (lengths up to 14336; longer ones use
  *                cuFFT in double), spreading and interpolation; the kernel
- *                values are stored as float pairs.  opts.fp64_contraction = 1
- *                and opts.fft_kernels = -1 together select FP64 instructions
+ *                values are stored as float pairs.  Spreading and interpolation
+ *                with 12 <= w <= 17 in 16-cell bins that hold at least 16
+ *                points run on the tensor cores instead: operands scaled per
+ *                tile to five base-1024 digits, exact fp16 products (2^-48 of
+ *                the scales), the kernel values along phi stored as digits.
+ *                opts.fp64_contraction = 1 and opts.fft_kernels = -1 together select FP64 instructions
  *                for every stage.  Measured eps_eff at lmax 4095 is ~6e-12
  *                either way, against the 1e-10 target.
  *   NUSHT_MIXED  coefficients complex64, maps float.  The Legendre recurrence,
@@ -128,7 +132,7 @@ typedef struct {
                          fast_recurrence = 1, and nusht_plan_many), every call for
                          NUSHT_FP64 plans; 1 = once at plan time; -1 = every call.  At plan
                          time the values are kept in device memory (a float per (ring pair,
-                         l, m) in mixed mode, a float pair in FP64 mode: 59 / 118 GB at lmax
+                         l, m) in mixed mode, a float pair in FP64 mode: 51 / 118 GB at lmax
                          4095) when they fit in half the free memory, else the recurrence
                          runs every call */
   int tensor_cores;   /* batched plans whose recurrence table fits: 0 (default) = the
@@ -137,9 +141,10 @@ typedef struct {
                          ~2^-21 relative per product); -1 = FP32 FMA on the CUDA cores */
   int fast_recurrence; /* 1 = run the P_lm recurrence of single-transform per-call plans in
                           double-float on the FP32 pipe (x, q_l, c_l as float pairs, ~2^-47
-                          relative per step instead of FP64's 2^-53; about 2.5x faster Legendre
-                          stages on GB300).  Opt-in: the default recurrence is FP64.  Ignored
-                          with fp64_contraction = 1 and in recurrence-table mode. */
+                          relative per step instead of FP64's 2^-53).  With the two-degree
+                          FP64 recurrence the default is the faster one for NUSHT_FP64
+                          plans; this one helps mixed plans with legendre_table = -1.
+                          Opt-in: the default recurrence is FP64.  Ignored with fp64_contraction = 1 and in recurrence-table mode. */
   int fft_kernels;    /* FP64 plans: 0 (default) = the theta FFT and the fine-grid 2D real FFT
                          run as this library's double-float kernels (one line per CTA in
                          shared memory, ~2^-47 relative per operation) when every length is
@@ -288,8 +293,8 @@ NUSHT_API int nusht_pointing(nusht_plan_t p, const void* d_philm, double* d_ptg,
  * entries are ignored.  The same chain as nusht_synth (Eq. SHTfast) with a
  * Wigner-d recurrence for S and the spin sign (-1)^s in the doubling.
  * Precision: the two Wigner-d recurrences (d^l_{m,-s}, d^l_{m,s}) in FP64
- * with scaled exponents, the sums over l in double-float (as the spin-0
- * Legendre contraction), the rest as in nusht_synth; measured eps_eff 7e-12
+ * from the step where each first reaches 2^-74 (found at plan time), the
+ * sums over l in double-float (as the spin-0 Legendre contraction), the rest as in nusht_synth; measured eps_eff 7e-12
  * at lmax 4095 against the 1e-10 target.
  *   d_glm, d_clm  device complex128[nalm]
  *   d_q, d_u      device double[npts], caller's point order

@@ -19,6 +19,10 @@
 // not accumulated; ring blocks of an order whose every ring stays below that
 // threshold up to lmax are dropped from the work list at plan time.
 //
+// The one-degree kernels below serve fp64_contraction, fast_recurrence, the FP64
+// recurrence table and mixed plans that run the recurrence in every call; FP64
+// plans run legendre2.cu and mixed plans legtab.cu by default.
+//
 // Parallel layout: one warp per work item (order m, block of 128 ring pairs),
 // four ring pairs (theta_j, pi - theta_j) per lane that share the recurrence
 // through Pbar_l(pi - theta) = (-1)^(l+m) Pbar_l(theta).

@@ -961,7 +961,7 @@ __global__ void __launch_bounds__(128) spread_pt_k(float* __restrict__ grid, int
 // always lie in 32 banks.  Taps beyond w have weight 0 and stay inside the tile's padding.
 // What bounds it is the shared-memory pipe and issue: two loads and two stores
 // of the tile and two 8-byte loads of weights per point, the same for every w.
-// 32 uniform sets of lmax 256 to 1535, w 7, 60M points: 4.33 -> 2.82 ms.
+// 32 uniform sets of lmax 256 to 1535, w 7, about 60M points: 4.33 -> 2.73 ms.
 constexpr int SW_PT = 28;  // words per staged point: 4 (p1, p1') and 8 (p2, cell) pairs, padded
 constexpr int SW_WMIN = 6, SW_WMAX = 8;
 __host__ __device__ inline int sw_stride(int binsz) { return (binsz + 30) / 32 * 32 + 8; }
