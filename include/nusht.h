@@ -45,8 +45,8 @@
  *                points run on the tensor cores instead: operands scaled per
  *                tile to five base-1024 digits, exact fp16 products (2^-48 of
  *                the scales), the kernel values along phi stored as digits.
- *                opts.fp64_contraction = 1 and opts.fft_kernels = -1 together select FP64 instructions
- *                for every stage.  Measured eps_eff at lmax 4095 is ~6e-12
+ *                opts.fp64_contraction = 1 and opts.fft_kernels = -1 together
+ *                select FP64 instructions for every stage.  Measured eps_eff at lmax 4095 is ~6e-12
  *                either way, against the 1e-10 target.
  *   NUSHT_MIXED  coefficients complex64, maps float.  The Legendre recurrence,
  *                its rescaling and the DFS fold in double (by default the
@@ -144,7 +144,8 @@ typedef struct {
                           relative per step instead of FP64's 2^-53).  With the two-degree
                           FP64 recurrence the default is the faster one for NUSHT_FP64
                           plans; this one helps mixed plans with legendre_table = -1.
-                          Opt-in: the default recurrence is FP64.  Ignored with fp64_contraction = 1 and in recurrence-table mode. */
+                          Opt-in: the default recurrence is FP64.  Ignored with
+                          fp64_contraction = 1 and in recurrence-table mode. */
   int fft_kernels;    /* FP64 plans: 0 (default) = the theta FFT and the fine-grid 2D real FFT
                          run as this library's double-float kernels (one line per CTA in
                          shared memory, ~2^-47 relative per operation) when every length is
@@ -294,7 +295,8 @@ NUSHT_API int nusht_pointing(nusht_plan_t p, const void* d_philm, double* d_ptg,
  * Wigner-d recurrence for S and the spin sign (-1)^s in the doubling.
  * Precision: the two Wigner-d recurrences (d^l_{m,-s}, d^l_{m,s}) in FP64
  * from the step where each first reaches 2^-74 (found at plan time), the
- * sums over l in double-float (as the spin-0 Legendre contraction), the rest as in nusht_synth; measured eps_eff 7e-12
+ * sums over l in double-float (as the spin-0 Legendre contraction), the rest
+ * as in nusht_synth; measured eps_eff 7e-12
  * at lmax 4095 against the 1e-10 target.
  *   d_glm, d_clm  device complex128[nalm]
  *   d_q, d_u      device double[npts], caller's point order
