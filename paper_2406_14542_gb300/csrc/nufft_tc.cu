@@ -40,7 +40,6 @@
 #include "dfloat.cuh"
 #include "nusht_internal.cuh"
 #include "ozsplit.cuh"
-#include "recurrence.cuh"
 #include "tc_pack.cuh"
 
 namespace nusht {
@@ -147,6 +146,9 @@ __device__ __forceinline__ float2 levels(float s0, float s1, float s2, float s3,
   return make_float2(h, __fmaf_rn(__fmaf_rn(s4, 0x1p-10f, s3), 0x1p-30f, __fadd_rn(e1, e2)));
 }
 
+// Operands are scaled by oz_scale: a value so far below the largest that its
+// scaled exponent would leave the double range is zero (split_qr drops
+// everything below 2^-74 of the largest in any case).
 // The largest magnitude of an operand, as a double's high word without its
 // sign: 2^exp_of bounds it; below 2^-900 it counts as zero, from 2^128 on (an
 // infinity or NaN among them; the FFT stages' float pairs end there) the
@@ -209,8 +211,8 @@ __global__ void __launch_bounds__(128, 7) interp_tc_k(const double* __restrict__
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     float2 x, y;
-    split_qr(too_small(mx) ? 0.0 : rec::scale_pow2(u[k][0], -ue), x.x, x.y);
-    split_qr(too_small(mx) ? 0.0 : rec::scale_pow2(u[k][1], -ue), y.x, y.y);
+    split_qr(too_small(mx) ? 0.0 : oz_scale(u[k][0], -ue), x.x, x.y);
+    split_qr(too_small(mx) ? 0.0 : oz_scale(u[k][1], -ue), y.x, y.y);
     put_pairs(sm.U[0] + at(tr0 + 8 * k, tc), 32 * 32, x, y);
   }
   __syncthreads();
@@ -301,7 +303,7 @@ __global__ void __launch_bounds__(128, 7) interp_tc_k(const double* __restrict__
       }
     }
     if (t4 < 2 && g4 + 8 * t4 < np)
-      out[po] = rec::scale_pow2(df_value(t4 ? fh[1] : fh[0], t4 ? fl[1] : fl[0]), too_small(mx) ? 0 : ue - 18);
+      out[po] = oz_scale(df_value(t4 ? fh[1] : fh[0], t4 ? fl[1] : fl[0]), too_small(mx) ? 0 : ue - 18);
     __syncwarp();  // P is refilled by the next group
   }
 }
@@ -357,7 +359,7 @@ __global__ void __launch_bounds__(ST, 4) spread_tc_k(double* __restrict__ grid, 
   const int fe = exp_of(mx);
   for (int q = threadIdx.x; q < tot; q += ST) {  // a thread's own values
     float2 v;
-    split_qr(none ? 0.0 : rec::scale_pow2(reinterpret_cast<const double*>(sm.f)[q], -fe), v.x, v.y);
+    split_qr(none ? 0.0 : oz_scale(reinterpret_cast<const double*>(sm.f)[q], -fe), v.x, v.y);
     sm.f[q] = v;
   }
   const int m0 = (warp >> 2) * 16;

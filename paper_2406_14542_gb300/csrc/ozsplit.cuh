@@ -116,6 +116,14 @@ OZ_HD long long oz_fix_f(float v, int k) {
   return (b >> 31) ? -r : r;
 }
 
+// v 2^k through the exponent field; 0 where that is below the normal range and
+// for zero and subnormal v.  |v 2^k| < 2^1024, v finite.
+OZ_HD double oz_scale(double v, int k) {
+  const unsigned long long b = oz_bits_d(v);
+  const int ex = (int)(b >> 52) & 0x7ff;
+  return ex > 0 && ex + k > 0 ? oz_double_of(b + ((unsigned long long)(long long)k << 52)) : 0.0;
+}
+
 // N 2^k as a double (round half away from zero to 53 bits); results below
 // the normal range are 0
 OZ_HD double oz_dbl(long long N, int k) {
