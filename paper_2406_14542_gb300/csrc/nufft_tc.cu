@@ -21,11 +21,14 @@
 // digits, x = sum_i d_i 2^(-9 - 10 i) with integers |d_i| <= 528, each exact in
 // fp16.  mma.sync (fp16 operands, fp32 accumulation) forms the 15 digit
 // products with i + j <= 4; the products of one level i + j accumulate into one
-// fp32 sum, which holds integers exactly up to 2^24: w <= 17 nonzero terms per
-// product in interpolation, 32 points between two conversions to integer in
-// spreading.  What is dropped (level 5 on) is below 2^-48 of the operands' scales, the
-// largest value of the tile (of the subproblem's point values); the sum of the
-// levels is carried as a float pair or a 64-bit integer.
+// fp32 sum, which holds integers exactly up to 2^24.  Interpolation adds w <= 17
+// nonzero terms per product: levels 0 to 2 stay below 2^24, levels 3 and 4
+// (2^-48 and 2^-58 of the scales) may round their last bit.  Spreading adds any
+// number of points and moves what would outgrow 2^24 into integers
+// (tc_digits.cuh).  What is dropped (level 5 on) is below 2^-48 of the operands'
+// scales: the tile's largest grid value; the largest point value of a block, a
+// run of up to TC_RUN subproblems; the kernel's 1.  The sum of the levels is
+// carried as a float pair or a 64-bit integer.
 //
 // The warp-level MMA serves this shape: products of 16 points (or cells) by 8,
 // operands made by the warps that consume them at once.  At its 1024
@@ -40,6 +43,7 @@
 #include "dfloat.cuh"
 #include "nusht_internal.cuh"
 #include "ozsplit.cuh"
+#include "tc_digits.cuh"
 #include "tc_pack.cuh"
 
 namespace nusht {
@@ -47,7 +51,6 @@ namespace nusht {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int ND = 5;        // digits per operand
 constexpr int BIN = 16;      // bin edge the kernels are written for
 constexpr int TC_SUB = 256;  // most points of a subproblem
 constexpr int GP = 16;       // points per interpolation group (rows of one MMA)
@@ -77,20 +80,6 @@ __device__ __forceinline__ void put_packed(__half* dst, int stride, uint2 x, uin
   put(2, num(p2, 1536.f));
   put(3, num(p3, 1536.f));
   put(4, num(((p0 >> 10) & 0x001f001fu) | ((p1 >> 5) & 0x03e003e0u), 1536.f));
-}
-
-// x = h + l, |x| <= 1, |l| <= 2^-24 |h|: x = sum_i d[i] 2^(-9 - 10 i) + O(2^-50)
-__device__ __forceinline__ void digits(float h, float l, float d[ND]) {
-  constexpr float C = 12582912.0f;  // 1.5 2^23: adding and subtracting it rounds to an integer
-  float x = h * 512.0f;
-  d[0] = __fsub_rn(__fadd_rn(x, C), C);
-  x = (x - d[0]) * 1024.0f;
-  d[1] = __fsub_rn(__fadd_rn(x, C), C);
-  const float r = x - d[1], L = l * 536870912.0f;  // 2^29
-  d[2] = __fsub_rn(__fadd_rn(__fmaf_rn(r, 1024.0f, L), C), C);
-  x = __fadd_rn(__fmaf_rn(r, 1024.0f, -d[2]), L) * 1024.0f;
-  d[3] = __fsub_rn(__fadd_rn(x, C), C);
-  d[4] = __fsub_rn(__fadd_rn((x - d[3]) * 1024.0f, C), C);
 }
 
 // ... and from float pairs
@@ -315,8 +304,7 @@ __global__ void __launch_bounds__(128, 7) interp_tc_k(const double* __restrict__
 // new one, so the warps of the left half write their sums out and take the new
 // right half: a cell is added to the grid twice instead of four times.  32
 // points at a time are split into digits by the whole block, a pair of tile
-// rows and a pair of tile columns of one point per thread.  Levels 0 and 1 go to integers after every chunk (their fp32 sums are then at most 2^23
-// and 2^24); the higher levels weigh 2^-20 and less and stay in fp32.
+// rows and a pair of tile columns of one point per thread.
 // ---------------------------------------------------------------------------
 struct __align__(16) SpreadSmem {
   __half A[ND][CP * 32];             // f_p psi1_p, [point][tile row]
@@ -382,10 +370,7 @@ __global__ void __launch_bounds__(ST, 4) spread_tc_k(double* __restrict__ grid, 
     for (int c = 0; c < 4; ++c) {
       const int tr = m0 + (lane >> 2) + 8 * (c >> 1), tc = nn0 + 2 * (lane & 3) + (c & 1);
       if (tr >= tw || tc >= tw) continue;
-      // sum_s 2^(-18 - 10 s) level_s, in units of 2^-48
-      const long long v = ((long long)sum[0][c] << 30) + ((long long)sum[1][c] << 20) +
-                          ((long long)__float2int_rn(acc[2][c]) << 10) +
-                          (long long)__float2int_rn(__fmaf_rn(acc[4][c], 0x1p-10f, acc[3][c]));
+      const long long v = tc_total(sum[0][c], sum[1][c], acc[2][c], acc[3][c], acc[4][c]);
       const double x = bad ? quiet_nan() : oz_dbl(v, fe - 48);
       if (scratch) {
         float2 o;
@@ -437,14 +422,11 @@ __global__ void __launch_bounds__(ST, 4) spread_tc_k(double* __restrict__ grid, 
 #pragma unroll
           for (int j = 0; i + j < ND; ++j) mma(acc[i + j], A, B[j][0], B[j][1]);
         }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tc_carry2(acc[2][c], sum[1][c]);
       }
 #pragma unroll
-      for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          sum[s][c] += __float2int_rn(acc[s][c]);
-          acc[s][c] = 0.f;
-        }
+      for (int c = 0; c < 4; ++c) tc_carry(acc[0][c], acc[1][c], acc[2][c], acc[3][c], sum[0][c], sum[1][c]);
       __syncthreads();  // A and B are refilled by the next chunk
     }
     q0 += cnt;
