@@ -27,8 +27,11 @@
 // number of points and moves what would outgrow 2^24 into integers
 // (tc_digits.cuh).  What is dropped (level 5 on) is below 2^-48 of the operands'
 // scales: the tile's largest grid value; the largest point value of a block, a
-// run of up to TC_RUN subproblems; the kernel's 1.  The sum of the levels is
-// carried as a float pair or a 64-bit integer.
+// run of up to TC_RUN subproblems; the kernel's 1.  For the widest kernels
+// (FINE) level 5 is kept, its operands scaled by 2^-10 into level 4's sum, and
+// the values of a spreading block, which may lie far below their scale, have a
+// sixth digit.  The sum of the levels is carried as a float pair or a 64-bit
+// integer.
 //
 // The warp-level MMA serves this shape: products of 16 points (or cells) by 8,
 // operands made by the warps that consume them at once.  At its 1024
@@ -39,6 +42,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "dfloat.cuh"
 #include "nusht_internal.cuh"
@@ -82,13 +86,14 @@ __device__ __forceinline__ void put_packed(__half* dst, int stride, uint2 x, uin
   put(4, num(((p0 >> 10) & 0x001f001fu) | ((p1 >> 5) & 0x03e003e0u), 1536.f));
 }
 
-// ... and from float pairs
+// ... and N digits from float pairs
+template <int N>
 __device__ __forceinline__ void put_pairs(__half* dst, int stride, float2 x, float2 y) {
-  float dx[ND], dy[ND];
-  digits(x.x, x.y, dx);
-  digits(y.x, y.y, dy);
+  float dx[N], dy[N];
+  digits<N>(x.x, x.y, dx);
+  digits<N>(y.x, y.y, dy);
 #pragma unroll
-  for (int i = 0; i < ND; ++i) *reinterpret_cast<__half2*>(dst + i * stride) = __floats2half2_rn(dx[i], dy[i]);
+  for (int i = 0; i < N; ++i) *reinterpret_cast<__half2*>(dst + i * stride) = __floats2half2_rn(dx[i], dy[i]);
 }
 
 __device__ __forceinline__ void mma(float d[4], const unsigned a[4], unsigned b0, unsigned b1) {
@@ -96,6 +101,11 @@ __device__ __forceinline__ void mma(float d[4], const unsigned a[4], unsigned b0
       "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// two digits times 2^-10, still exact in fp16: their products go one level up
+__device__ __forceinline__ unsigned up_level(unsigned v) {
+  const __half2 h = __hmul2(*reinterpret_cast<__half2*>(&v), __float2half2_rn(0x1p-10f));
+  return *reinterpret_cast<const unsigned*>(&h);
 }
 __device__ __forceinline__ void ldm4(unsigned r[4], const __half* p) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -157,6 +167,7 @@ struct __align__(16) InterpSmem {
   int mx[4];
 };
 
+template <bool FINE>
 __global__ void __launch_bounds__(128, 7) interp_tc_k(const double* __restrict__ grid, int64_t stride, int n1, int n2,
                                                       int nb2, int w, float ipw, const int* __restrict__ sub,
                                                       const int* __restrict__ cell, const float2* __restrict__ psi,
@@ -202,7 +213,7 @@ __global__ void __launch_bounds__(128, 7) interp_tc_k(const double* __restrict__
     float2 x, y;
     split_qr(too_small(mx) ? 0.0 : oz_scale(u[k][0], -ue), x.x, x.y);
     split_qr(too_small(mx) ? 0.0 : oz_scale(u[k][1], -ue), y.x, y.y);
-    put_pairs(sm.U[0] + at(tr0 + 8 * k, tc), 32 * 32, x, y);
+    put_pairs<ND>(sm.U[0] + at(tr0 + 8 * k, tc), 32 * 32, x, y);
   }
   __syncthreads();
   __half* P = sm.P[warp][0];
@@ -272,6 +283,7 @@ __global__ void __launch_bounds__(128, 7) interp_tc_k(const double* __restrict__
           ldm2(B, sm.U[j] + at(min(n0 + (lane & 7), 31), ks * 16 + ((lane >> 3) & 1) * 8));
 #pragma unroll
           for (int i = 0; i + j < ND; ++i) mma(acc[i + j], A[i], B[0], B[1]);
+          if (FINE && j > 0) mma(acc[ND - 1], A[ND - j], up_level(B[0]), up_level(B[1]));
         }
       }
 #pragma unroll
@@ -306,8 +318,9 @@ __global__ void __launch_bounds__(128, 7) interp_tc_k(const double* __restrict__
 // points at a time are split into digits by the whole block, a pair of tile
 // rows and a pair of tile columns of one point per thread.
 // ---------------------------------------------------------------------------
+template <int NA>
 struct __align__(16) SpreadSmem {
-  __half A[ND][CP * 32];             // f_p psi1_p, [point][tile row]
+  __half A[NA][CP * 32];             // f_p psi1_p, [point][tile row]
   __half B[ND][CP * 32];             // psi2_p, [point][tile column]
   float2 f[TC_RUN * TC_SUB];         // the run's values (scaled, as float pairs)
   unsigned char cell[TC_RUN * TC_SUB];  // and first taps, 16 (row) + column
@@ -315,13 +328,15 @@ struct __align__(16) SpreadSmem {
   int mx[ST / 32];
 };
 
+template <bool FINE>
 __global__ void __launch_bounds__(ST, 4) spread_tc_k(double* __restrict__ grid, int64_t stride, int n1, int n2,
                                                       int nb2, int w, float ipw, const int* __restrict__ sub, int nsub,
                                                       int run, const int* __restrict__ cell,
                                                       const float2* __restrict__ psi, const int* __restrict__ perm,
                                                       const double* __restrict__ f, float2* __restrict__ scratch) {
+  constexpr int NA = FINE ? ND + 1 : ND;  // digits of f_p psi1_p
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  SpreadSmem& sm = *reinterpret_cast<SpreadSmem*>(smem_raw);
+  SpreadSmem<NA>& sm = *reinterpret_cast<SpreadSmem<NA>*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i0 = blockIdx.x * run, ni = min(run, nsub - i0);
   if ((int)threadIdx.x < 3 * ni) sm.sub[threadIdx.x] = sub[3 * i0 + threadIdx.x];
@@ -371,7 +386,7 @@ __global__ void __launch_bounds__(ST, 4) spread_tc_k(double* __restrict__ grid, 
       const int tr = m0 + (lane >> 2) + 8 * (c >> 1), tc = nn0 + 2 * (lane & 3) + (c & 1);
       if (tr >= tw || tc >= tw) continue;
       const long long v = tc_total(sum[0][c], sum[1][c], acc[2][c], acc[3][c], acc[4][c]);
-      const double x = bad ? quiet_nan() : oz_dbl(v, fe - 48);
+      const double x = bad ? quiet_nan() : oz_dbl(v, fe - 51);
       if (scratch) {
         float2 o;
         df_of(x, o.x, o.y);
@@ -393,7 +408,7 @@ __global__ void __launch_bounds__(ST, 4) spread_tc_k(double* __restrict__ grid, 
     for (int p0 = q0; p0 < q0 + cnt; p0 += CP) {
       const int np = min(CP, q0 + cnt - p0);
       float4* z = reinterpret_cast<float4*>(sm.A[0]);
-      for (int t = threadIdx.x; t < 2 * ND * CP * 4; t += ST) z[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int t = threadIdx.x; t < (NA + ND) * CP * 4; t += ST) z[t] = make_float4(0.f, 0.f, 0.f, 0.f);
       __syncthreads();
       for (int t = threadIdx.x; t < np * npw; t += ST) {
         const int p = __float2int_rz(((float)t + 0.5f) * ipw);  // t / npw, as in interp_tc_k
@@ -407,7 +422,7 @@ __global__ void __launch_bounds__(ST, 4) spread_tc_k(double* __restrict__ grid, 
         const uint2 xb = b >= 0 && b < w ? __ldg(pk + b) : TC_ZERO, yb = b + 1 < w ? __ldg(pk + b + 1) : TC_ZERO;
         const float2 fp = sm.f[p0 + p];
         put_packed(sm.B[0] + at(p, cc + b), CP * 32, xb, yb);
-        put_pairs(sm.A[0] + at(p, cr + a), CP * 32, df_mul(x, fp), df_mul(y, fp));
+        put_pairs<NA>(sm.A[0] + at(p, cr + a), CP * 32, df_mul(x, fp), df_mul(y, fp));
       }
       __syncthreads();
       for (int ks = 0; ks * 16 < np; ++ks) {
@@ -416,11 +431,12 @@ __global__ void __launch_bounds__(ST, 4) spread_tc_k(double* __restrict__ grid, 
         for (int j = 0; j < ND; ++j)
           ldm2t(B[j], sm.B[j] + at(ks * 16 + ((lane >> 3) & 1) * 8 + (lane & 7), nn0));
 #pragma unroll
-        for (int i = 0; i < ND; ++i) {
+        for (int i = 0; i < NA; ++i) {
           unsigned A[4];
           ldm4t(A, sm.A[i] + at(ks * 16 + (lane >> 4) * 8 + (lane & 7), m0 + ((lane >> 3) & 1) * 8));
 #pragma unroll
           for (int j = 0; i + j < ND; ++j) mma(acc[i + j], A, B[j][0], B[j][1]);
+          if (FINE && i > 0) mma(acc[ND - 1], A, up_level(B[ND - i][0]), up_level(B[ND - i][1]));
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c) tc_carry2(acc[2][c], sum[1][c]);
@@ -458,17 +474,41 @@ bool nufft_tc(nusht_plan_t p) {
          p->sz.w <= 17 && d.npts >= (int64_t)TC_FILL * d.nsub;
 }
 
+// Whether level 5 is kept, by the spreading kernel's own error, about
+// e^(-pi w sqrt(1 - 1 / sigma)).  Without it the digits lose 2^-48 of their
+// scales, which the deconvolution raises to 1e-13 of an adjoint (2.5e-13 where
+// the values of a block span six decades): more than float pairs, and to be
+// seen beside a kernel error below 1e-12 (w = 16 at sigma 1.5: adjoint of such a
+// map, lmax 200, against 128-bit sums: float pairs 6.7e-13, without level 5
+// 6.9e-13, with it 6.6e-13; w = 17: 1.30e-13, 2.77e-13, 1.31e-13).  It costs 2.1M
+// points at lmax 1023, w = 17 interpolation 338 -> 360 us, spreading 439 -> 485.
+constexpr double TC_FINE = 1e-12;
+static bool fine_products(nusht_plan_t p) {
+  return std::exp(-M_PI * p->sz.w * std::sqrt(1.0 - 1.0 / p->sz.sigma)) < TC_FINE;
+}
+
 int tc_smem_optin() {
-  NUSHT_CUDA(cudaFuncSetAttribute(interp_tc_k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(InterpSmem)));
-  NUSHT_CUDA(cudaFuncSetAttribute(spread_tc_k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SpreadSmem)));
+  auto set = [](auto k, size_t n) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+  };
+  NUSHT_CUDA(set(interp_tc_k<false>, sizeof(InterpSmem)));
+  NUSHT_CUDA(set(interp_tc_k<true>, sizeof(InterpSmem)));
+  NUSHT_CUDA(set(spread_tc_k<false>, sizeof(SpreadSmem<ND>)));
+  NUSHT_CUDA(set(spread_tc_k<true>, sizeof(SpreadSmem<ND + 1>)));
   return NUSHT_OK;
 }
 
 int tc_interp(nusht_plan_t p, double* d_map, cudaStream_t s) {
   const nusht_sizes& z = p->sz;
-  interp_tc_k<<<p->pts.nsub, 128, sizeof(InterpSmem), s>>>(
-      (const double*)p->fine, 2 * (z.n2 / 2 + 1), z.n1, z.n2, p->pts.nbins2, z.w, 1.0f / (float)((z.w + 2) / 2), p->pts.sub,
-      p->pts.cell, reinterpret_cast<const float2*>(p->pts.psi), p->pts.perm, d_map);
+  auto go = [&](auto k, size_t sm) {
+    k<<<p->pts.nsub, 128, sm, s>>>((const double*)p->fine, 2 * (z.n2 / 2 + 1), z.n1, z.n2, p->pts.nbins2, z.w,
+                                   1.0f / (float)((z.w + 2) / 2), p->pts.sub, p->pts.cell,
+                                   reinterpret_cast<const float2*>(p->pts.psi), p->pts.perm, d_map);
+  };
+  if (fine_products(p))
+    go(interp_tc_k<true>, sizeof(InterpSmem));
+  else
+    go(interp_tc_k<false>, sizeof(InterpSmem));
   NUSHT_CUDA(cudaGetLastError());
   return NUSHT_OK;
 }
@@ -478,9 +518,16 @@ int tc_spread(nusht_plan_t p, const double* d_map, float2* tiles, cudaStream_t s
   // runs as long as three waves of blocks remain; one subproblem per block
   // where each tile is wanted by itself
   const int run = tiles ? 1 : std::max(1, std::min(TC_RUN, p->pts.nsub / (3 * 4 * 152)));
-  spread_tc_k<<<(p->pts.nsub + run - 1) / run, ST, sizeof(SpreadSmem), s>>>(
-      (double*)p->fine, 2 * (z.n2 / 2 + 1), z.n1, z.n2, p->pts.nbins2, z.w, 1.0f / (float)((z.w + 2) / 2), p->pts.sub,
-      p->pts.nsub, run, p->pts.cell, reinterpret_cast<const float2*>(p->pts.psi), p->pts.perm, d_map, tiles);
+  auto go = [&](auto k, size_t sm) {
+    k<<<(p->pts.nsub + run - 1) / run, ST, sm, s>>>(
+        (double*)p->fine, 2 * (z.n2 / 2 + 1), z.n1, z.n2, p->pts.nbins2, z.w, 1.0f / (float)((z.w + 2) / 2),
+        p->pts.sub, p->pts.nsub, run, p->pts.cell, reinterpret_cast<const float2*>(p->pts.psi), p->pts.perm, d_map,
+        tiles);
+  };
+  if (fine_products(p))
+    go(spread_tc_k<true>, sizeof(SpreadSmem<ND + 1>));
+  else
+    go(spread_tc_k<false>, sizeof(SpreadSmem<ND>));
   NUSHT_CUDA(cudaGetLastError());
   return NUSHT_OK;
 }

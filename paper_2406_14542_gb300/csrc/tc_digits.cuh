@@ -5,11 +5,14 @@
 
 namespace nusht {
 
-constexpr int ND = 5;  // digits per operand
+constexpr int ND = 5;  // digits per operand, levels of products
 
-// x = h + l, |x| <= 1, |l| <= 2^-24 |h|: x = sum_i d[i] 2^(-9 - 10 i) + O(2^-50)
-// with integers |d[i]| <= 512 (d[2]: 528, it takes the leading part of l)
-__device__ __forceinline__ void digits(float h, float l, float d[ND]) {
+// x = h + l, |x| <= 1, |l| <= 2^-24 |h|, in N = 5 or 6 digits:
+// x = sum_i d[i] 2^(-9 - 10 i) + O(2^-50), with six O(2^-54) (the low bits of a
+// pair far below 1 are rounded on the way), with integers |d[i]| <= 512 (d[2]:
+// 528, it takes the leading part of l)
+template <int N>
+__device__ __forceinline__ void digits(float h, float l, float d[N]) {
   constexpr float C = 12582912.0f;  // 1.5 2^23: adding and subtracting it rounds to an integer
   float x = h * 512.0f;
   d[0] = __fsub_rn(__fadd_rn(x, C), C);
@@ -19,7 +22,9 @@ __device__ __forceinline__ void digits(float h, float l, float d[ND]) {
   d[2] = __fsub_rn(__fadd_rn(__fmaf_rn(r, 1024.0f, L), C), C);
   x = __fadd_rn(__fmaf_rn(r, 1024.0f, -d[2]), L) * 1024.0f;
   d[3] = __fsub_rn(__fadd_rn(x, C), C);
-  d[4] = __fsub_rn(__fadd_rn((x - d[3]) * 1024.0f, C), C);
+  x = (x - d[3]) * 1024.0f;
+  d[4] = __fsub_rn(__fadd_rn(x, C), C);
+  if (N > 5) d[5] = __fsub_rn(__fadd_rn((x - d[4]) * 1024.0f, C), C);
 }
 
 // One cell of a spreading tile: the fp32 sums s[i + j] of the products a_i b_j
@@ -48,10 +53,11 @@ __device__ __forceinline__ void tc_carry(float& s0, float& s1, float& s2, float&
   s0 = s1 = 0.0f;
   s2 += __fsub_rn(tc_over(s3), 12582912.0f);
 }
-// sum_s 2^(-18 - 10 s) level_s in units of 2^-48
+// sum_s 2^(-18 - 10 s) level_s in units of 2^-51: 2,303 products of at most 1,
+// the most a tile holds, stay below 2^63
 __device__ __forceinline__ long long tc_total(int n0, int n1, float s2, float s3, float s4) {
-  return ((long long)n0 << 30) + ((long long)n1 << 20) + ((long long)__float2int_rn(s2) << 10) +
-         (long long)__float2int_rn(__fmaf_rn(s4, 0x1p-10f, s3));
+  return ((long long)n0 << 33) + ((long long)n1 << 23) + ((long long)__float2int_rn(s2) << 13) +
+         (long long)__float2int_rn(__fmaf_rn(s4, 0x1p-7f, s3 * 8.0f));
 }
 
 }  // namespace nusht

@@ -13,7 +13,9 @@ here with g++ (the few CUDA intrinsics they use are given as plain C++).
   random ones.  Against the exact sum of the kept digit products the total is
   off by at most 16 units of 2^-48 per 32 points (level 3, four MMAs per 16
   points, each losing less than two units above 2^24) and two units of the
-  last conversion.
+  last conversion.  Against the sum of the operands' products each point may
+  lose 2^-47 (the dropped products and digits) or, with level 5 and six digits
+  of one operand, 2^-50 of the other's missing digit and 2^-54 of its own.
 """
 import os
 import shutil
@@ -99,10 +101,9 @@ using namespace nusht;
 typedef __int128 big;
 
 // an fp32 accumulator after the exact sum x
-static float acc32(long long x, bool truncate) {
-  float f = (float)x;
-  if (truncate && std::llabs((long long)f) > std::llabs(x)) f = std::nextafterf(f, 0.0f);
-  return f;
+static float acc32(double x, bool truncate) {
+  const float f = (float)x;
+  return truncate && std::fabs((double)f) > std::fabs(x) ? std::nextafterf(f, 0.0f) : f;
 }
 static void digits_of_psi(double psi, int d[5]) {
   const uint2 v = tc_pack(psi);
@@ -120,37 +121,49 @@ int main() {
   long bad = 0;
   for (int n : {1, 16, 31, 256, 672, 2303})
     for (int kind = 0; kind < 20; ++kind)
-      for (int truncate = 0; truncate < 2; ++truncate) {
-        const double x0 = kind == 0 ? top : U(g), p0 = kind == 0 ? top : U(g);
-        float s[ND] = {};
-        int n0 = 0, n1 = 0;
-        big exact = 0;
-        for (int q0 = 0; q0 < n; q0 += 32) {
-          for (int k0 = q0; k0 < std::min(n, q0 + 32); k0 += 16) {
-            long long lev[ND][ND] = {};
-            for (int q = k0; q < std::min(n, k0 + 16); ++q) {
-              const double x = kind < 14 ? x0 : (kind < 17 ? 1.0 : (g() & 1 ? 1 : -1)) * U(g), p = kind < 14 ? p0 : U(g);
-              float h, l, a[ND];
-              int b[5];
-              split_qr(x, h, l);
-              digits(h, l, a);
-              digits_of_psi(p, b);
-              for (int i = 0; i < ND; ++i)
-                for (int j = 0; i + j < ND; ++j) {
-                  lev[i][j] += (long long)a[i] * b[j];
-                  exact += (big)((long long)a[i] * b[j]) << (10 * (ND - 1 - i - j));
-                }
+      for (int truncate = 0; truncate < 2; ++truncate)
+        for (int fine = 0; fine < 2; ++fine) {
+          const double x0 = kind == 0 ? top : U(g), p0 = kind == 0 ? top : U(g);
+          float s[ND] = {};
+          int n0 = 0, n1 = 0;
+          big kept = 0;  // in units of 2^-68
+          long double all = 0;
+          for (int q0 = 0; q0 < n; q0 += 32) {
+            for (int k0 = q0; k0 < std::min(n, q0 + 32); k0 += 16) {
+              long long lev[ND + 1] = {};
+              for (int q = k0; q < std::min(n, k0 + 16); ++q) {
+                double x = kind < 14 ? x0 : (kind < 17 ? 1.0 : (g() & 1 ? 1 : -1)) * U(g), p = kind < 14 ? p0 : U(g);
+                if (kind > 10 && q % 3) x *= 0x1p-20;
+                float h, l, a[ND + 1] = {};
+                int b[5];
+                split_qr(x, h, l);
+                if (fine)
+                  digits<ND + 1>(h, l, a);
+                else
+                  digits<ND>(h, l, a);
+                digits_of_psi(p, b);
+                for (int i = 0; i < ND + fine; ++i)
+                  for (int j = 0; j < ND && i + j < ND + fine; ++j) {
+                    lev[i + j] += (long long)a[i] * b[j];
+                    kept += (big)((long long)a[i] * b[j]) << (10 * (ND - i - j));
+                  }
+                all += ((long double)h + (long double)l) * (long double)p;
+              }
+              for (int k = 0; k < ND; ++k) {
+                // level 5 joins level 4 times 2^-10
+                const double v = (double)s[k] + (double)lev[k] + (k == ND - 1 ? (double)lev[ND] * 0x1p-10 : 0.0);
+                s[k] = acc32(v, truncate);
+              }
+              tc_carry2(s[2], n1);
             }
-            for (int i = 0; i < ND; ++i)
-              for (int j = 0; i + j < ND; ++j) s[i + j] = acc32((long long)s[i + j] + lev[i][j], truncate);
-            tc_carry2(s[2], n1);
+            tc_carry(s[0], s[1], s[2], s[3], n0, n1);
           }
-          tc_carry(s[0], s[1], s[2], s[3], n0, n1);
+          const long long got = tc_total(n0, n1, s[2], s[3], s[4]);  // 2^-51
+          const long double rounding = 0x1p-48L * (16 * ((n + 31) / 32) + 2);
+          if (std::fabs((long double)(((big)got << 17) - kept)) * 0x1p-68L > rounding) ++bad;
+          const long double lost = n * (fine ? 0x1p-50L + 0x1p-54L : 0x1p-47L);
+          if (std::fabs((long double)got * 0x1p-51L - all) > rounding + lost) ++bad;
         }
-        const big got = (big)tc_total(n0, n1, s[2], s[3], s[4]) << (10 * (ND - 4));
-        const big off = got > exact ? got - exact : exact - got;
-        if (off > ((big)(16 * ((n + 31) / 32) + 2) << (10 * (ND - 4)))) ++bad;
-      }
   std::printf("%ld\n", bad);
   return bad != 0;
 }
