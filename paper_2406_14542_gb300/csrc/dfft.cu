@@ -955,19 +955,28 @@ bool wide(const DfftLen& f) {
   return true;
 }
 
-// Threads of a line kernel (compiled for tmax a block).  The registers allow
-// tmax threads on an SM: as many shorter blocks as the lines' shared memory
-// allows share them, so that one line's barriers do not idle the whole SM, as
-// long as a thread keeps about three radix-4 butterflies a pass.  All six
-// passes of a step, 1024 threads a line -> this rule: lines of 2048 and 3072
-// (lmax 1023, now 256 threads) 705 -> 453 us, of 4096 and 6144 (lmax 2047, now
-// 512) 2.55 -> 1.95 ms.  The row passes with a radix 5 or 7 keep their 512
-// threads (13.3 us against 14.8 with 256 at 1568 values, their column passes
-// 21.8 -> 16.5): their strided reads of T want the warps.
-int line_threads(const DfftLen& f, int tmax) {
+// Threads of a line kernel (compiled for tmax a block) on `lines` lines.
+//  * Not more than a radix-4 butterfly a pass each, but 256: the others would
+//    only wait at the barriers (lines of 256 and 384 values, lmax 127: 66 us a
+//    step with 1024 threads, 61 with 512, 60 with 256, 64 with 128, 76 with 64).
+//  * The registers allow tmax threads on an SM.  Where there are more lines than
+//    such blocks, as many shorter blocks as the lines' shared memory allows share
+//    an SM, so that one line's barriers do not idle it, as long as a thread
+//    keeps about three butterflies a pass, up to four blocks.  Six passes of a
+//    step, 1024 threads a line -> this rule: lines of 2048 and 3072 (lmax 1023,
+//    now 256 threads) 705 -> 453 us, of 4096 and 6144 (lmax 2047, now 512) 2.55
+//    -> 1.95 ms; odd radices at lmax 400: 512 threads 190 us, 256 184, 128 159.
+//    With fewer lines shorter blocks only make each line slower (lines of 512
+//    and 768, lmax 255 with 77 orders: 107 us a step with 64 threads, 69 with 256).
+// The row passes with a radix 5 or 7 keep their 512 threads (13.3 us against
+// 14.8 with 256 at 1568 values, their column passes 21.8 -> 16.5): their strided
+// reads of T want the warps.
+int line_threads(nusht_plan_t p, const DfftLen& f, int lines, int tmax) {
   const int fit = SFFT_SMEM_MAX / (f.N * (int)sizeof(float4));
   int t = tmax;
-  while (t > 64 && 2 * (tmax / t) <= fit && f.N <= 12 * (t / 2)) t /= 2;
+  while ((t > 256 && f.N <= 4 * (t / 2)) ||
+         (t > tmax / 4 && f.N <= 12 * (t / 2) && 2 * (tmax / t) <= fit && lines > p->sms * (tmax / t)))
+    t /= 2;
   return t;
 }
 
@@ -1067,9 +1076,9 @@ int dfft_theta_exec(nusht_plan_t p, const void* src, void* dst, int sign, cudaSt
   const DfftLen& f = p->dft_theta;
   auto go = [&](auto kw, auto ko) {
     if (wide(f))
-      kw<<<nl, line_threads(f, DFFT_T_WIDE), sm, s>>>(src, dst, z.M, nl, f);
+      kw<<<nl, line_threads(p, f, nl, DFFT_T_WIDE), sm, s>>>(src, dst, z.M, nl, f);
     else
-      ko<<<nl, line_threads(f, DFFT_T_ODD), sm, s>>>(src, dst, z.M, nl, f);
+      ko<<<nl, line_threads(p, f, nl, DFFT_T_ODD), sm, s>>>(src, dst, z.M, nl, f);
   };
   if (sign < 0) {
     if (p->dfft_fine)
@@ -1094,9 +1103,9 @@ int dfft_theta_pairs(nusht_plan_t p, const void* src, void* dst, int sign, cudaS
   const DfftLen& f = p->dft_theta;
   auto go = [&](auto kw, auto ko) {
     if (wide(f))
-      kw<<<nl, line_threads(f, DFFT_T_WIDE), sm, s>>>(src, dst, z.M, nl, f);
+      kw<<<nl, line_threads(p, f, nl, DFFT_T_WIDE), sm, s>>>(src, dst, z.M, nl, f);
     else
-      ko<<<nl, line_threads(f, DFFT_T_ODD), sm, s>>>(src, dst, z.M, nl, f);
+      ko<<<nl, line_threads(p, f, nl, DFFT_T_ODD), sm, s>>>(src, dst, z.M, nl, f);
   };
   if (sign < 0)
     go(dfft_lines_k<-1, true, true, DFFT_T_WIDE>, dfft_lines_k<-1, true, true, DFFT_T_ODD>);
@@ -1109,14 +1118,15 @@ int dfft_theta_pairs(nusht_plan_t p, const void* src, void* dst, int sign, cudaS
 int dfft_cols_synth(nusht_plan_t p, cudaStream_t s) {
   const nusht_sizes& z = p->sz;
   const size_t sm = (size_t)dline_words(z.n1) * sizeof(float4);
+  const int nl = z.mmax + 1;
   const DfftLen& f = p->dft_n1;
   auto go = [&](auto kw, auto ko) {
     if (wide(f))
-      kw<<<z.mmax + 1, line_threads(f, DFFT_T_WIDE), sm, s>>>(p->Ghat, (float4*)p->tcols, z.lmax, z.M, p->deconv1f, p->deconv2f, f,
-                                             p->pts.rowmask);
+      kw<<<nl, line_threads(p, f, nl, DFFT_T_WIDE), sm, s>>>(p->Ghat, (float4*)p->tcols, z.lmax, z.M, p->deconv1f,
+                                                             p->deconv2f, f, p->pts.rowmask);
     else
-      ko<<<z.mmax + 1, line_threads(f, DFFT_T_ODD), sm, s>>>(p->Ghat, (float4*)p->tcols, z.lmax, z.M, p->deconv1f, p->deconv2f, f,
-                                            p->pts.rowmask);
+      ko<<<nl, line_threads(p, f, nl, DFFT_T_ODD), sm, s>>>(p->Ghat, (float4*)p->tcols, z.lmax, z.M, p->deconv1f,
+                                                            p->deconv2f, f, p->pts.rowmask);
   };
   if (p->dfft_theta)
     go(dfft_cols_synth_k<true, DFFT_T_WIDE>, dfft_cols_synth_k<true, DFFT_T_ODD>);
@@ -1134,8 +1144,8 @@ int dfft_rows_c2r(nusht_plan_t p, cudaStream_t s) {
   const int np = p->pts.nrowpairs;  // only the row pairs some point reaches
   if (np == 0) return NUSHT_OK;
   if (wide(f))
-    dfft_rows_c2r_k<DFFT_T_WIDE><<<np, line_threads(f, DFFT_T_WIDE), sm, s>>>((const float4*)p->tcols, (double*)p->fine, stride, z.n1,
-                                                            z.mmax, f, p->pts.rowpairs);
+    dfft_rows_c2r_k<DFFT_T_WIDE><<<np, line_threads(p, f, np, DFFT_T_WIDE), sm, s>>>(
+        (const float4*)p->tcols, (double*)p->fine, stride, z.n1, z.mmax, f, p->pts.rowpairs);
   else
     dfft_rows_c2r_k<DFFT_T_ODD><<<np, DFFT_T_ODD, sm, s>>>((const float4*)p->tcols, (double*)p->fine, stride, z.n1,
                                                           z.mmax, f, p->pts.rowpairs);
@@ -1151,8 +1161,8 @@ int dfft_rows_r2c(nusht_plan_t p, cudaStream_t s) {
   const int np = p->pts.nrowpairs;  // rows no point reaches stay zero: their spectra in T are zero
   if (np == 0) return NUSHT_OK;
   if (wide(f))
-    dfft_rows_r2c_k<DFFT_T_WIDE><<<np, line_threads(f, DFFT_T_WIDE), sm, s>>>((const double*)p->fine, (float4*)p->tcols, stride,
-                                                            z.n1, z.mmax, f, p->pts.rowpairs);
+    dfft_rows_r2c_k<DFFT_T_WIDE><<<np, line_threads(p, f, np, DFFT_T_WIDE), sm, s>>>(
+        (const double*)p->fine, (float4*)p->tcols, stride, z.n1, z.mmax, f, p->pts.rowpairs);
   else
     dfft_rows_r2c_k<DFFT_T_ODD><<<np, DFFT_T_ODD, sm, s>>>((const double*)p->fine, (float4*)p->tcols, stride, z.n1,
                                                           z.mmax, f, p->pts.rowpairs);
@@ -1163,14 +1173,15 @@ int dfft_rows_r2c(nusht_plan_t p, cudaStream_t s) {
 int dfft_cols_adjoint(nusht_plan_t p, cudaStream_t s) {
   const nusht_sizes& z = p->sz;
   const size_t sm = (size_t)dline_words(z.n1) * sizeof(float4);
+  const int nl = z.mmax + 1;
   const DfftLen& f = p->dft_n1;
   auto go = [&](auto kw, auto ko) {
     if (wide(f))
-      kw<<<z.mmax + 1, line_threads(f, DFFT_T_WIDE), sm, s>>>((const float4*)p->tcols, p->Ghat, z.lmax, z.M, p->deconv1f,
-                                             p->deconv2f, f, p->pts.rowmask);
+      kw<<<nl, line_threads(p, f, nl, DFFT_T_WIDE), sm, s>>>((const float4*)p->tcols, p->Ghat, z.lmax, z.M,
+                                                             p->deconv1f, p->deconv2f, f, p->pts.rowmask);
     else
-      ko<<<z.mmax + 1, line_threads(f, DFFT_T_ODD), sm, s>>>((const float4*)p->tcols, p->Ghat, z.lmax, z.M, p->deconv1f,
-                                            p->deconv2f, f, p->pts.rowmask);
+      ko<<<nl, line_threads(p, f, nl, DFFT_T_ODD), sm, s>>>((const float4*)p->tcols, p->Ghat, z.lmax, z.M,
+                                                            p->deconv1f, p->deconv2f, f, p->pts.rowmask);
   };
   if (p->dfft_theta)
     go(dfft_cols_adj_k<true, DFFT_T_WIDE>, dfft_cols_adj_k<true, DFFT_T_ODD>);

@@ -255,6 +255,7 @@ struct StageEvents {
 
 struct nusht_plan_s {
   int device = 0;
+  int sms = 0;  // streaming multiprocessors of the device
   int lmax = 0, mmax = 0, precision = NUSHT_FP64;
   double eps = 0.0;
   nusht_sizes sz{};

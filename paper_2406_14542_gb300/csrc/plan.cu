@@ -337,7 +337,7 @@ int nusht::fine_fft_r2c(nusht_plan_t p, cudaStream_t s) {
   return NUSHT_OK;
 }
 
-static int check_device(int* dev) {
+static int check_device(int* dev, int* sms) {
   int n = 0;
   cudaError_t e = cudaGetDeviceCount(&n);
   if (e != cudaSuccess || n == 0) {
@@ -349,6 +349,7 @@ static int check_device(int* dev) {
   NUSHT_CUDA(cudaGetDeviceProperties(&prop, *dev));
   if (!(prop.major == 10 && prop.minor == 3))
     return set_error(NUSHT_EDEVICE, std::string("library is built for sm_103a (GB300); device is ") + prop.name);
+  *sms = prop.multiProcessorCount;
   return NUSHT_OK;
 }
 
@@ -457,14 +458,15 @@ int nusht::plan_create(nusht_plan_t* out, int lmax, int mmax, int64_t npts, cons
   if (opts && (opts->spin < 0 || opts->spin > lmax)) return set_error(NUSHT_EINVAL, "spin must be in [0, lmax]");
   if (opts && opts->spin > 0 && (precision != NUSHT_FP64 || !role.legendre || !role.nufft))
     return set_error(NUSHT_EUNSUPPORTED, "spin transforms need a standalone NUSHT_FP64 plan");
-  int dev = 0;
-  NUSHT_TRY(check_device(&dev));
+  int dev = 0, sms = 0;
+  NUSHT_TRY(check_device(&dev, &sms));
   const char* fa = std::getenv("NUSHT_FAIL_ALLOC_AFTER");
   g_fail_after = fa ? std::atol(fa) : -1;
   g_alloc_count = 0;
   nusht_plan_t p = new (std::nothrow) nusht_plan_s();
   if (!p) return set_error(NUSHT_ENOMEM, "host allocation failed");
   p->device = dev;
+  p->sms = sms;
   p->lmax = lmax;
   p->mmax = mmax;
   p->precision = precision;
