@@ -462,16 +462,29 @@ __global__ void __launch_bounds__(ST, 4) spread_tc_k(double* __restrict__ grid, 
 
 }  // namespace
 
-// Whether the plan's interpolation and spreading run on the tensor cores:
-// tiles of 32 cells (16-cell bins, w <= 17), kernels wide enough and bins full
-// enough for the dense products to pay.  Interpolation + spreading, float
-// pairs against this file, 2.1M points at lmax 1023 (112 points a bin):
-// w = 9 538 : 760 us, w = 12 735 : 650, w = 14 862 : 645, w = 17 1166 : 800;
-// with 11 points a bin w = 12 201 : 250, w = 14 237 : 252, w = 17 307 : 273.
+// Whether the plan's interpolation and spreading run on the tensor cores: tiles
+// of 32 cells (16-cell bins, w <= 17), kernels wide enough and bins full enough
+// (points per subproblem, on average) for the dense products to pay.  Float
+// pairs : this file, interpolation + spreading in us, uniform points, lmax 1023
+// (18,400 bins):
+//   points a bin      16          26          38          64
+//   w = 12        248 : 293   303 : 334   369 : 376   503 : 478
+//   w = 13        260 : 296   318 : 336   384 : 380   519 : 481
+//   w = 14        287 : 301   352 : 339   426 : 386   584 : 492
+//   w = 15        329 : 304   404 : 342   491 : 389   674 : 501
+// (w = 9, 112 points: 538 : 760).  A few thousand bins do not fill the device, and
+// the shorter blocks of this file hide their latency better: at lmax 383 (2,600
+// bins, 16 points) w = 12 takes 61 : 56 us, w = 14 65 : 59; at lmax 511 (4,600) 80
+// : 82 and 89 : 86, with 38 points 112 : 106 and 131 : 112.
+constexpr int TC_WMIN = 12;
+static int tc_fill(nusht_plan_t p) {
+  const int w = p->sz.w;
+  return p->pts.nsub <= 32 * p->sms || w > 14 ? 16 : w == 14 ? 20 : w == 13 ? 32 : 40;
+}
 bool nufft_tc(nusht_plan_t p) {
   const PointData& d = p->pts;
   return p->precision == NUSHT_FP64 && !p->opts.fp64_contraction && d.bin == BIN && p->sz.w >= TC_WMIN &&
-         p->sz.w <= 17 && d.npts >= (int64_t)TC_FILL * d.nsub;
+         p->sz.w <= 17 && d.npts >= (int64_t)tc_fill(p) * d.nsub;
 }
 
 // Whether level 5 is kept, by the spreading kernel's own error, about
@@ -517,7 +530,7 @@ int tc_spread(nusht_plan_t p, const double* d_map, float2* tiles, cudaStream_t s
   const nusht_sizes& z = p->sz;
   // runs as long as three waves of blocks remain; one subproblem per block
   // where each tile is wanted by itself
-  const int run = tiles ? 1 : std::max(1, std::min(TC_RUN, p->pts.nsub / (3 * 4 * 152)));
+  const int run = tiles ? 1 : std::max(1, std::min(TC_RUN, p->pts.nsub / (3 * 4 * p->sms)));
   auto go = [&](auto k, size_t sm) {
     k<<<(p->pts.nsub + run - 1) / run, ST, sm, s>>>(
         (double*)p->fine, 2 * (z.n2 / 2 + 1), z.n1, z.n2, p->pts.nbins2, z.w, 1.0f / (float)((z.w + 2) / 2),

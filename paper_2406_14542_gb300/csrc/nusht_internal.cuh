@@ -383,8 +383,6 @@ int spread(nusht_plan_t p, const void* d_map, cudaStream_t s);
 int spread_smem_optin();
 // the same on the tensor cores (nufft_tc.cu): whether a plan's point set takes
 // that path, shared-memory opt-in, execution (tiles: deterministic mode)
-constexpr int TC_WMIN = 12;  // narrower kernels: float pairs
-constexpr int TC_FILL = 16;  // fewer points per subproblem on average: float pairs
 bool nufft_tc(nusht_plan_t p);
 int tc_smem_optin();
 int tc_interp(nusht_plan_t p, double* d_map, cudaStream_t s);
