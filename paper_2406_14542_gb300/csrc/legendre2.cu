@@ -472,6 +472,7 @@ __global__ void __launch_bounds__(128, 6) leg2_adj_k(Leg2Args a, const int* __re
     __syncwarp();  // the slots are rewritten by the next four steps
     if (half == 0 && d < 2 * ns) reinterpret_cast<float2*>(out + 2 * base + d)[cpt] = make_float2(sh, sl);
   }
+  if (STAGED) copies_wait<0>();  // the chunk past the last one
 }
 
 // c_lm from the block partials (summed as float pairs in a fixed order, only

@@ -328,6 +328,7 @@ __global__ void __launch_bounds__(128) spin_synth_k(SpinArgs a, const float4* __
     }
     __syncwarp();
   }
+  copies_wait<0>();  // the chunk past the last one
   if (jn > a.npairs) return;
   const double sgs = (s & 1) ? -1.0 : 1.0;               // (-1)^s
   const double sgd = ((m + s) & 1) ? -1.0 : 1.0;         // doubling sign (-1)^(m+s)
@@ -535,6 +536,7 @@ __global__ void __launch_bounds__(128) spin_adj_k(SpinArgs a, const double2* __r
     }
     __syncwarp();
   }
+  copies_wait<0>();  // the chunk past the last one
 }
 
 // c_lm = s_l times the sum over the partial rows of the groups that have
