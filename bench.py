@@ -461,14 +461,15 @@ def main():
                "extrapolated": True,
                "sample": "%d seeded points (synthesis + adjoint over all orders), scaled by N/%d; "
                          "the direct sum is exactly linear in N" % (nsample, nsample)}
-    # synthesis: leg2_coef, leg2_synth, theta DFT, column pass, row pass, interp_df;
-    # adjoint: spread_df, row pass, column pass, theta DFT, leg2_adj, leg2_reduce
+    # synthesis: leg2_coef, leg2_synth, theta DFT, column pass, row pass, interp_tc;
+    # adjoint: spread_tc, row pass, column pass, theta DFT, leg2_adj, leg2_reduce
     launches_per_step = 12
     line = {
         "metric": METRIC, "value": fp["ms"] / world, "unit": "ms", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": fp["ms"], "higher_is_better": False, "scaling": "weak",
         "vs_baseline": None,
-        "dtype": "f64 recurrence; double-float (float pairs, ~2^-47 per op) contraction, FFTs, NUFFT",
+        "dtype": "f64 recurrence; double-float (float pairs, ~2^-47 per op) contraction, FFTs; NUFFT: exact fp16 "
+                 "digit products to 2^-48 of the operands' scales",
         "data": "synthetic",
         "config": {"workload": "deflected GL grid %dx%d (%d pts), lmax=mmax=%d, "
                                "C_l=(l+1)^-2 Gaussian a_lm, 2.5 arcmin rms deflection" % (L + 1, 2 * L + 1, npts, L),
@@ -638,8 +639,8 @@ def run_spin(torch, nu, args, dist, rank, L, pts):
     return {"ms_per_step": ms, "synth_ms": e[0].elapsed_time(e[1]), "adjoint_ms": e[1].elapsed_time(e[2]),
             "eps_eff": par, "eps_eff_sample": 200, "plan_s": t_plan, "plan_GB": nbytes / 1e9, "spin": 2,
             "what": "FP64 Wigner-d recurrences (both +-s chains per ring pair), float-pair sums on the FP32 pipe, "
-                    "passes whose values stay below 2^-300 skipped; theta FFT, fine-grid FFT and NUFFT once per "
-                    "field (Q, U)", "clocks": clk.summary()}
+                    "each chain from the degree where it first reaches 2^-74; theta FFT, fine-grid FFT and NUFFT once "
+                    "per field (Q, U)", "clocks": clk.summary()}
 
 
 def run_autograd(torch, nu, args, dist):
@@ -789,7 +790,7 @@ def _kernel_hash() -> str:
     import hashlib
 
     h = hashlib.sha1()
-    for f in ("legendre.cu", "legendre2.cu", "recurrence.cuh", "dfloat.cuh"):
+    for f in ("legendre2.cu", "recurrence.cuh", "dfloat.cuh", "async_copy.cuh"):
         with open(os.path.join(ROOT, "paper_2406_14542_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:12]

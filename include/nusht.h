@@ -41,13 +41,17 @@
  *                and the fine-grid 2D FFT (lengths up to 14336; longer ones use
  *                cuFFT in double), spreading and interpolation; the kernel
  *                values are stored as float pairs.  Spreading and interpolation
- *                with 12 <= w <= 17 in 16-cell bins that hold at least 16
- *                points run on the tensor cores instead: operands scaled per
- *                tile to five base-1024 digits, exact fp16 products (2^-48 of
- *                the scales), the kernel values along phi stored as digits.
+ *                with 12 <= w <= 17 in 16-cell bins run on the tensor cores
+ *                instead where the bins hold enough points on average (16, with
+ *                thousands of bins 40, 32 and 20 for w = 12, 13 and 14):
+ *                operands as base-1024 digits and exact fp16 products, to 2^-48
+ *                of the tile's largest grid value and of the largest point
+ *                value of up to eight bins (finer where the kernel's own error
+ *                is below 1e-12), the kernel values along phi stored as digits;
+ *                a NaN, an infinity or a value from 2^128 on among them gives NaN.
  *                opts.fp64_contraction = 1 and opts.fft_kernels = -1 together
- *                select FP64 instructions for every stage.  Measured eps_eff at lmax 4095 is ~6e-12
- *                either way, against the 1e-10 target.
+ *                select FP64 instructions for every stage.  Measured eps_eff at
+ *                lmax 4095 is ~6e-12 either way, against the 1e-10 target.
  *   NUSHT_MIXED  coefficients complex64, maps float.  The Legendre recurrence,
  *                its rescaling and the DFS fold in double (by default the
  *                recurrence runs once at plan time, see opts.legendre_table);

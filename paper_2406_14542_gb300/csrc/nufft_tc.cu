@@ -9,13 +9,12 @@
 // The float-pair kernels (nufft.cu) spend 13 FP32 instructions on each of a
 // point's w^2 taps; here the taps are tensor-core work and a point costs the
 // splitting of its 2 w kernel values and, in interpolation, w float-pair
-// multiply-adds: about 100 warp instructions a point instead of 150
-// (interpolation) and 220 (spreading) at w = 14.  At lmax 1023 (2.1M points)
-// interpolation 329 -> 282 us, spreading 534 -> 362; at lmax 4095 (33.6M)
-// 5.08 -> 4.38 and 8.00 -> 5.44 ms; 20,000 points at lmax 63: 15 -> 12 and
-// 68 -> 12 us.  What bounds both is issue (62 and 54 % of the slots) and the
-// latency of the points' reads and of the block's phases; the tensor pipe is
-// idle four fifths of the time.
+// multiply-adds: about 100 (interpolation) and 125 (spreading) warp instructions
+// a point instead of 150 and 220 at w = 14.  At lmax 1023 (2.1M points)
+// interpolation 329 -> 285 us, spreading 534 -> 378; at lmax 4095 (33.6M) 5.08
+// -> 4.43 and 8.00 -> 5.69 ms.  What bounds both is issue (62 and 59 % of the
+// slots) and the latency of the points' reads and of the block's phases; the
+// tensor pipe is idle three quarters of the time.
 //
 // Exact products.  An operand scaled to |x| <= 1 is written in five balanced
 // digits, x = sum_i d_i 2^(-9 - 10 i) with integers |d_i| <= 528, each exact in
@@ -311,8 +310,8 @@ __global__ void __launch_bounds__(128, 7) interp_tc_k(const double* __restrict__
 
 // ---------------------------------------------------------------------------
 // spreading: a block takes a run of consecutive subproblems (mostly bins next
-// to each other along phi).  Each of the eight warps owns 16 x 8 cells of the tile;
-// moving one bin on, the right half of the old tile is the left half of the
+// to each other along phi).  Each of the eight warps owns 16 x 8 cells of the
+// tile; moving one bin on, the right half of the old tile is the left half of the
 // new one, so the warps of the left half write their sums out and take the new
 // right half: a cell is added to the grid twice instead of four times.  32
 // points at a time are split into digits by the whole block, a pair of tile

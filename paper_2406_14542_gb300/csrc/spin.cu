@@ -540,10 +540,13 @@ __global__ void __launch_bounds__(128) spin_adj_k(SpinArgs a, const double2* __r
 }
 
 // c_lm = s_l times the sum over the partial rows of the groups that have
-// started at degree l, in a fixed order (float pairs), plus the poles (order s); entries with l < s are 0, Im of the m = 0 entries is 0
+// started at degree l, in a fixed order (float pairs), plus the poles (order
+// s); entries with l < s are 0, Im of the m = 0 entries is 0
 __global__ void spin_adj_reduce_k(const float4* __restrict__ pg, const float4* __restrict__ pc,
-                                  const int* __restrict__ gst, const double* __restrict__ scl, int nrows, int64_t nalm, int L, int mmax, int s, int M, const double2* __restrict__ HQ,
-                                  const double2* __restrict__ HU, double2* __restrict__ og, double2* __restrict__ oc) {
+                                  const int* __restrict__ gst, const double* __restrict__ scl, int nrows,
+                                  int64_t nalm, int L, int mmax, int s, int M, const double2* __restrict__ HQ,
+                                  const double2* __restrict__ HU, double2* __restrict__ og,
+                                  double2* __restrict__ oc) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nalm) return;
   // (l, m) of packed index i: order m holds l = m..L at m (2L + 1 - m) / 2 + l,
@@ -727,8 +730,8 @@ void spin_free(nusht_plan_t p) {
 int spin_legendre_synth(nusht_plan_t p, const void* glm, const void* clm, cudaStream_t s) {
   const SpinArgs a = spin_args(p);
   const int nitems = (p->mmax + 1) * a.ngrp;
-  spin_scale_k<<<(int)((p->nalm + 255) / 256), 256, 0, s>>>((const double2*)glm, (const double2*)clm,
-                                                             p->spin.sc, p->nalm, p->lmax, p->opts.spin, p->spin.ap, p->spin.am);
+  spin_scale_k<<<(int)((p->nalm + 255) / 256), 256, 0, s>>>((const double2*)glm, (const double2*)clm, p->spin.sc,
+                                                             p->nalm, p->lmax, p->opts.spin, p->spin.ap, p->spin.am);
   spin_synth_k<<<(nitems + 3) / 4, 128, 0, s>>>(a, p->spin.ap, p->spin.am, p->spin.GQ, p->spin.GU);
   spin_poles_k<<<1, 256, 0, s>>>(p->lmax, p->mmax, p->opts.spin, p->sz.M, (const double2*)glm, (const double2*)clm,
                                  p->spin.GQ, p->spin.GU);

@@ -18,7 +18,8 @@ namespace nusht {
 
 __host__ __device__ __forceinline__ uint2 tc_pack(double psi) {
   // 512 in every field below the first makes the digits unsigned
-  const long long y = (long long)(psi * 0x1p59 + 0.5) + 512ll * (1 + (1ll << 10) + (1ll << 20) + (1ll << 30) + (1ll << 40));
+  const long long low = 512ll * (1 + (1ll << 10) + (1ll << 20) + (1ll << 30) + (1ll << 40));
+  const long long y = (long long)(psi * 0x1p59 + 0.5) + low;
   auto f = [&](int i) { return (unsigned)(y >> (10 * (5 - i))) & (i ? 1023u : 0xffffu); };
   return make_uint2(f(0) | (f(4) & 31u) << 10 | (f(1) | (f(4) >> 5) << 10) << 16,
                     f(2) | (f(5) & 31u) << 10 | (f(3) | (f(5) >> 5) << 10) << 16);

@@ -37,7 +37,13 @@ inline uint2 make_uint2(unsigned x, unsigned y) { return {x, y}; }
 #define __forceinline__ inline
 struct float2 { float x, y; };
 inline float2 make_float2(float x, float y) { return {x, y}; }
-template <class T, class F> inline T bits_as(F v) { T r; static_assert(sizeof(T) == sizeof(F), ""); std::memcpy(&r, &v, sizeof r); return r; }
+template <class T, class F>
+inline T bits_as(F v) {
+  static_assert(sizeof(T) == sizeof(F), "");
+  T r;
+  std::memcpy(&r, &v, sizeof r);
+  return r;
+}
 inline int __double2hiint(double v) { return (int)(bits_as<uint64_t>(v) >> 32); }
 inline int __double2loint(double v) { return (int)(uint32_t)bits_as<uint64_t>(v); }
 inline float __uint_as_float(unsigned v) { return bits_as<float>(v); }
